@@ -673,8 +673,8 @@ ct_status ct_load_state(const ct_case* c, int precision, void* work, const void*
   return launch_dt(c, precision, work, U, cfl, st, uses_prims(c, precision));
 }
 
-// CTAs of a launch of the surrogate queue kernel: two per SM, what its registers and shared
-// memory are budgeted for (persistent; the queue's length is known on the device only).
+// CTAs of a launch of the surrogate queue kernel: one per SM, which its shared memory fills
+// (persistent; the queue's length is known on the device only).
 // The kernel never waits on another CTA, so CTAs beyond those resident only start later.
 static std::mutex g_qgrid_mu;
 static int g_qgrid[64];
@@ -685,7 +685,7 @@ static int queue_grid() {
   if (g_qgrid[dev] == 0) {
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) return 0;
-    g_qgrid[dev] = std::min(QUEUE_GRID_MAX, 2 * nsm);
+    g_qgrid[dev] = std::min(QUEUE_GRID_MAX, nsm);
   }
   return g_qgrid[dev];
 }
@@ -708,12 +708,8 @@ static ct_status set_stage_attrs(int shape, int p) {
       e = cudaFuncSetAttribute(ss->stage_sp[st], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss->smem[p]);
     if (e == cudaSuccess && p == 2 && ss->queue[st])
       e = cudaFuncSetAttribute(ss->queue[st], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss->queue_smem);
-    if (e == cudaSuccess && p == 2 && ss->queue[st])   // two CTAs per SM need most of the SM's shared memory
-      e = cudaFuncSetAttribute(ss->queue[st], cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e == cudaSuccess && p == 2 && ss->batch_queue[st])
       e = cudaFuncSetAttribute(ss->batch_queue[st], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss->queue_smem);
-    if (e == cudaSuccess && p == 2 && ss->batch_queue[st])
-      e = cudaFuncSetAttribute(ss->batch_queue[st], cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   }
   if (e != cudaSuccess) return fail(CT_ERR_CUDA, cudaGetErrorString(e));
   if (p == 2 && ss->queue[0] && queue_grid() <= 0)

@@ -401,38 +401,36 @@ __device__ inline void publish_stage(WsHeader* h, const double* fin, int stage, 
 }
 
 // ---- the fused stage kernel ---------------------------------------------------------------
-// shared memory of the surrogate phase, reusing the (then dead) stencil buffers:
-// activations, streamed weights, outputs, blob header, per-thread results
-constexpr size_t SM_A = 0, SM_W = SM_A + mlp::ABYTES, SM_OUT = SM_W + 32768, SM_HDR = SM_OUT + 128 * 10 * 4,
-                 SM_RES = SM_HDR + mlp::NFLOAT * 4;
-// the surrogate queue kernel of the column sweep (stage_sweep.cuh): threads, shared memory,
+// shared memory of the surrogate phase, reusing the (then dead) stencil buffers: activations of two
+// 128-row tiles (the outputs of their rows over them at the end), streamed weights
+constexpr size_t SM_A = 0, SM_W = SM_A + 2 * mlp::ABYTES, SM_SURR = SM_W + 32768;
+// the surrogate queue kernel of the column sweep (stage_sweep.cuh): threads (warpgroups of 128, each
+// on its own 128 cells), shared memory (all weights and an operand buffer per group),
 // CTAs of a launch at most (the room of its partial records in the workspace)
 struct QueueTile {
-  static constexpr int NT = 256;
+  static constexpr int NT = 128 * mlp::GROUPS;
 };
-constexpr size_t QUEUE_SMEM = SM_RES + (size_t)QueueTile::NT * 40;
+constexpr size_t QUEUE_SMEM = mlp::GROUP_SMEM;
 constexpr int QUEUE_GRID_MAX = 4096;
 template <class TL>
 constexpr size_t stage_smem_surr() {
-  return TL::template smem<float>() > SM_RES + (size_t)TL::NT * 40 ? TL::template smem<float>()
-                                                                     : SM_RES + (size_t)TL::NT * 40;
+  return TL::template smem<float>() > SM_SURR ? TL::template smem<float>() : SM_SURR;
 }
 
-// Tensor-core resources of a CTA: 128 TMEM columns and the MMA-completion mbarrier (outside
-// the overlaid stencil buffers).  The stage kernels take them once at the start
-// (ready = true); the surrogate routine can also take and free them around a single call
-// (ready = false), since a CTA that has relinquished its allocation permit may not
-// allocate again.
+// Tensor-core resources of a CTA: 256 TMEM columns and the MMA-completion mbarrier (outside
+// the overlaid stencil buffers).  The stage kernels take them once at the start, since a CTA that
+// has relinquished its allocation permit may not allocate again.
 static __shared__ uint64_t s_tc_mbar;   // MMA completion
 static __shared__ uint64_t s_tc_wbar;   // weight bulk copies
 static __shared__ uint32_t s_tc_slot;
+static __shared__ __align__(16) float s_tc_hdr[mlp::NFLOAT];   // the blob's header (hdr_entry)
 struct TcCtx {
   uint32_t tmem, phase, wphase;
-  bool ready;
 };
-__device__ __forceinline__ uint32_t tc_acquire() {
+__device__ __forceinline__ uint32_t tc_acquire(const unsigned char* __restrict__ blob) {
+  for (int q = threadIdx.x; q < mlp::NFLOAT; q += blockDim.x) s_tc_hdr[q] = mlp::hdr_entry(q, __ldg(reinterpret_cast<const float*>(blob) + q));
   if ((threadIdx.x >> 5) == 0) {
-    tc::tmem_alloc(tc::smem_addr(&s_tc_slot), 128);
+    tc::tmem_alloc(tc::smem_addr(&s_tc_slot), 256);
     tc::tmem_relinquish();
   }
   if (threadIdx.x == 0) {
@@ -449,37 +447,27 @@ __device__ __forceinline__ void tc_release(uint32_t tmem) {
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(tmem, 128);
+  if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(tmem, 256);
 }
 
 // Surrogate cells of one tile (called by all threads, only when the tile has at least one):
-// compaction into 128-row tiles and the BF16 tensor-core network.  Each surrogate cell's
-// thread finds its 10 outputs (raw units, held to the training range of their targets) in
-// res[10 * threadIdx.x ...] afterwards.  x: the cell's 16 raw inputs (kind == 2 only).
+// compaction into 128-row tiles, two at a time, and the BF16 tensor-core network.  Each surrogate
+// cell's thread gets its 10 outputs (raw units, held to the training range of their targets) in y.
+// x: the cell's 16 raw inputs (kind == 2 only).
 template <class TL>
-__device__ __noinline__ void surrogate_tile(const unsigned char* __restrict__ blob, int kind, const float* x,
+__device__ __noinline__ void surrogate_tile(const unsigned char* __restrict__ blob, int kind, const float* x, float* y,
                                             int& ntimeout, unsigned char* smem, TcCtx* tcx) {
   constexpr int NT = TL::NT;
   __shared__ int wcnt[NT / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float* ghdr = reinterpret_cast<const float*>(blob);
+  const float* hdr = s_tc_hdr;
   const unsigned mask = __ballot_sync(0xffffffffu, kind == 2);
   if (lane == 0) wcnt[warp] = __popc(mask);
   unsigned char* A = smem + SM_A;
   unsigned char* W = smem + SM_W;
-  float* outs = reinterpret_cast<float*>(smem + SM_OUT);
-  float* hdr = reinterpret_cast<float*>(smem + SM_HDR);
-  float* res = reinterpret_cast<float*>(smem + SM_RES);
-  for (int q = tid; q < mlp::NFLOAT; q += NT) hdr[q] = ghdr[q];
-  uint32_t tmem, phase = 0, wphase = 0;
-  if (tcx->ready) {
-    tmem = tcx->tmem;
-    phase = tcx->phase;
-    wphase = tcx->wphase;
-    __syncthreads();
-  } else {
-    tmem = tc_acquire();   // includes the barrier
-  }
+  float* outs = reinterpret_cast<float*>(A);
+  if (tid == 0) mlp::fetch_layer(W, blob + mlp::WOFF, 0, tc::smem_addr(&s_tc_wbar));
+  __syncthreads();
   int off = 0, total = 0;
   for (int w2 = 0; w2 < NT / 32; ++w2) {
     off += w2 < warp ? wcnt[w2] : 0;
@@ -487,18 +475,18 @@ __device__ __noinline__ void surrogate_tile(const unsigned char* __restrict__ bl
   }
   const int row = off + __popc(mask & ((1u << lane) - 1u));
   bool ok = true;
-  for (int c0 = 0; c0 < total; c0 += 128) {
-    const bool mine = kind == 2 && row >= c0 && row < c0 + 128;
+  for (int c0 = 0; c0 < total; c0 += 256) {
+    const bool mine = kind == 2 && row >= c0 && row < c0 + 256;
     if (mine) {
       float v[16];
 #pragma unroll
       for (int q = 0; q < 16; ++q) v[q] = (x[q] - hdr[mlp::F_XMEAN + q]) * hdr[mlp::F_XISD + q];
-      mlp::store_row16(A, row - c0, 0, 16, v);
+      mlp::store_row16(A + (row - c0 >= 128 ? mlp::ABYTES : 0), (row - c0) & 127, 0, 16, v);
     }
     float o[10];
-    ok = mlp::run_tile<true>(A, W, hdr + mlp::F_BIAS, tmem, tc::smem_addr(&s_tc_mbar), phase, o, blob + mlp::WOFF,
-                             total - c0, tc::smem_addr(&s_tc_wbar), &wphase) && ok;
-    if (tid < 128) {
+    ok = mlp::run_tiles(A, W, hdr + mlp::F_BIAS, tcx->tmem, tc::smem_addr(&s_tc_mbar), tcx->phase, o, blob + mlp::WOFF,
+                        total - c0, tc::smem_addr(&s_tc_wbar), &tcx->wphase, c0 + 256 < total) && ok;
+    if (tid < (total - c0 > 128 ? 256 : 128)) {   // over the activations, which the last product has read
 #pragma unroll
       for (int q = 0; q < 10; ++q) outs[tid * 10 + q] = o[q] * hdr[mlp::F_YSD + q] + hdr[mlp::F_YMEAN + q];
     }
@@ -506,89 +494,121 @@ __device__ __noinline__ void surrogate_tile(const unsigned char* __restrict__ bl
     if (mine) {
 #pragma unroll
       for (int q = 0; q < 10; ++q)
-        res[tid * 10 + q] = fminf(fmaxf(outs[(row - c0) * 10 + q], hdr[mlp::F_YMIN + q]), hdr[mlp::F_YMAX + q]);
+        y[q] = fminf(fmaxf(outs[(row - c0) * 10 + q], hdr[mlp::F_YMIN + q]), hdr[mlp::F_YMAX + q]);
     }
     __syncthreads();
-  }
-  if (tcx->ready) {
-    tcx->phase = phase;
-    tcx->wphase = wphase;
-  } else {
-    tc_release(tmem);
   }
   if (!ok && tid == 0) ntimeout += 1;   // a tensor-core wait gave up: the step reports it
 }
 
-// Source of the FP32 + surrogate path (called by all threads): active cells inside the
-// surrogate's training hull take their rates from the network, the others the plain source
-// (counted as fallbacks); both feed the plain path's tail, so conservation and the limiters
-// are exact.  Adds the source to acc.
-template <class TL, class T>
-__device__ __forceinline__ void surrogate_source(const DevCase& dc, const unsigned char* __restrict__ blob, bool cell,
-                                                 const Prim<T>& w, const T* u14, T* acc, T dt, int& nactive,
-                                                 int& nfallback, int& ntimeout, T& lnJh, T& lnJt,
-                                                 unsigned char* smem, TcCtx* tcx) {
-  const float* ghdr = reinterpret_cast<const float*>(blob);
-  int kind = 0;   // 0 inactive, 1 plain source (outside the hull), 2 surrogate
-  Sat<T> st;
-  st.lnSl = st.lnSi = st.lnpv = 0.0;
-  st.pres_l = st.pres_s = st.active = false;
-  T Q[NF];
+// Source of the FP32 + surrogate path: active cells inside the surrogate's training hull take
+// their rates from the network, the others the plain source (counted as fallbacks); both feed the
+// plain path's tail, so conservation and the limiters are exact.  In three parts, so that the
+// fused tile and the queue kernel run the network each in its own way between them.
+// What stays with the cell over the network's run:
+template <class T>
+struct SurrCell {
+  int kind;   // 0 inactive, 1 plain source (outside the hull), 2 surrogate
+  bool pres_l, pres_s;
+  double lnSl, lnSi;
+  T lnpv, lnJh, lnJt;
+};
+// saturation, inputs (x) and hull test; the plain source of a cell outside the hull, added to acc
+template <class T>
+__device__ __forceinline__ void surrogate_begin(const DevCase& dc, const float* hdr, bool cell, const Prim<T>& w, const T* u14,
+                                                T* acc, T dt, SurrCell<T>& c, float* x, int& nfallback) {
+  c.kind = 0;
+  c.pres_l = c.pres_s = false;
+  c.lnSl = c.lnSi = 0.0;
+  c.lnpv = T(0);
+  c.lnJh = c.lnJt = T(-INFINITY);
+  if (!cell || !dc.sc.phase_change) return;
+  bool pl, ps;
+  if (!populations(w, pl, ps) && clearly_inactive(w)) return;
+  const Sat<T> st = saturation(w, dc.sc);
+  if (!st.active) return;
+  mlp_features<T>(w, st, dc.sc.rp2, x);
+  bool inside = true;
 #pragma unroll
-  for (int f = 0; f < NF; ++f) Q[f] = T(0);
-  double lnJ2[2] = {-INFINITY, -INFINITY};
-  float x[CT_MLP_IN];
-  if (cell && dc.sc.phase_change) {
-    bool pl, ps;
-    const bool pops = populations(w, pl, ps);
-    if (pops || !clearly_inactive(w)) {
-      st = saturation(w, dc.sc);
-      if (st.active) {
-        mlp_features<T>(w, st, dc.sc.rp2, x);
-        bool inside = true;
-#pragma unroll
-        for (int q = 0; q < CT_MLP_IN; ++q)
-          inside = inside && x[q] >= ghdr[mlp::F_HMIN + q] && x[q] <= ghdr[mlp::F_HMAX + q];
-        kind = inside ? 2 : 1;
-      }
-    }
-  }
-  if (kind == 1) {
+  for (int q = 0; q < CT_MLP_IN; ++q) inside = inside && x[q] >= hdr[mlp::F_HMIN + q] && x[q] <= hdr[mlp::F_HMAX + q];
+  c.kind = inside ? 2 : 1;
+  c.pres_l = st.pres_l;
+  c.pres_s = st.pres_s;
+  c.lnSl = st.lnSl;
+  c.lnSi = st.lnSi;
+  c.lnpv = T(st.lnpv);
+  if (!inside) {
+    T Q[NF];
+    double lnJ2[2] = {-INFINITY, -INFINITY};
     const Rates<T> r = plain_rates<T>(w, st, dc.sc, lnJ2, nullptr, nullptr);
     source_tail<T>(w, u14, acc, dt, dc.sc, st.pres_l, st.pres_s, st.lnSl, st.lnSi, r, Q, nullptr);
+#pragma unroll
+    for (int f = 4; f < 13; ++f) acc[f] = rn_add(acc[f], Q[f]);   // never fused with the product in Q
+    c.lnJh = T(lnJ2[0]);
+    c.lnJt = T(lnJ2[1]);
     nfallback = 1;
   }
-  // the stencil buffers are dead from here on; tiles without a surrogate cell skip the rest
-  if (__syncthreads_or(kind == 2)) {
-    surrogate_tile<TL>(blob, kind, x, ntimeout, smem, tcx);
-    if (kind == 2) {
-      const float* y = reinterpret_cast<const float*>(smem + SM_RES) + 10 * threadIdx.x;
-      const bool nuc = st.lnSl > 0.0;
-      Rates<T> r;
-      r.Jeff = r.rc_um = T(0);
-      if (nuc) {
-        // nucleation is the plain path's closed form: the rates and the Kelvin radius of
-        // Eqs. 3, 4, 10 (exponent in FP64) and the Kantrowitz factor of Eq. 5 (T_sat by the
-        // Newton iteration, Young's law at r_crit); the network supplies growth and relaxation
-        const Cnt c = cnt_rates<T>(w, st.lnSl, dc.sc, lnJ2);
-        const T Tsat_l = prop_tsat<T, false>(dc.sc, T(st.lnpv));
-        const T phi = kantrowitz_phi<T>(w, gas_props<T>(w), c.rc, c.rhov, Tsat_l);
-        r.Jeff = T(c.Jsum) / (T(1) + phi);
-        r.rc_um = T(c.rc * 1e6);
-      }
-      r.Gl = st.pres_l ? T(MLP_G0 * sinhf(y[2])) : T(0);
-      r.Gs = st.pres_s ? T(MLP_G0 * sinhf(y[3])) : T(0);
-      r.xl = st.pres_l ? T(__expf(y[4])) : T(0);
-      r.xs = st.pres_s ? T(__expf(y[5])) : T(0);
-      source_tail<T>(w, u14, acc, dt, dc.sc, st.pres_l, st.pres_s, st.lnSl, st.lnSi, r, Q, nullptr);
+}
+// the source of a surrogate cell from its network outputs y, added to acc
+template <class T>
+__device__ __forceinline__ void surrogate_end(const DevCase& dc, const Prim<T>& w, const T* u14, T* acc, T dt, const float* y,
+                                              SurrCell<T>& c) {
+  Rates<T> r;
+  r.Jeff = r.rc_um = T(0);
+  if (c.lnSl > 0.0) {
+    // nucleation is the plain path's closed form: the rates and the Kelvin radius of
+    // Eqs. 3, 4, 10 (exponent in FP64) and the Kantrowitz factor of Eq. 5 (T_sat by the
+    // Newton iteration, Young's law at r_crit); the network supplies growth and relaxation
+    double lnJ2[2] = {-INFINITY, -INFINITY};
+    const Cnt n = cnt_rates<T>(w, c.lnSl, dc.sc, lnJ2);
+    const T Tsat_l = prop_tsat<T, false>(dc.sc, c.lnpv);
+    const T phi = kantrowitz_phi<T>(w, gas_props<T>(w), n.rc, n.rhov, Tsat_l);
+    r.Jeff = T(n.Jsum) / (T(1) + phi);
+    r.rc_um = T(n.rc * 1e6);
+    c.lnJh = T(lnJ2[0]);
+    c.lnJt = T(lnJ2[1]);
+  }
+  r.Gl = c.pres_l ? T(MLP_G0 * sinhf(y[2])) : T(0);
+  r.Gs = c.pres_s ? T(MLP_G0 * sinhf(y[3])) : T(0);
+  r.xl = c.pres_l ? T(__expf(y[4])) : T(0);
+  r.xs = c.pres_s ? T(__expf(y[5])) : T(0);
+  T Q[NF];
+  source_tail<T>(w, u14, acc, dt, dc.sc, c.pres_l, c.pres_s, c.lnSl, c.lnSi, r, Q, nullptr);
+#pragma unroll
+  for (int f = 4; f < 13; ++f) acc[f] = rn_add(acc[f], Q[f]);   // never fused with the product in Q
+}
+// The fused tile's form (called by all threads of the CTA).  u14 is taken from memory again
+// (U, plane stride N, cell n) and the primitives from it after the network's run: kept over the
+// call, they and the source's state made 400 bytes of stack per thread, more than the L1 left
+// beside two CTAs' shared memory holds.
+template <class TL, class T>
+__device__ __forceinline__ void surrogate_source(const DevCase& dc, const unsigned char* __restrict__ blob, bool cell,
+                                                 const Prim<T>& w, const T* __restrict__ U, size_t N, size_t n, T* u14, T* acc,
+                                                 T dt, int& nactive, int& nfallback, int& ntimeout, T& lnJh, T& lnJt,
+                                                 unsigned char* smem, TcCtx* tcx) {
+  SurrCell<T> c;
+  float x[CT_MLP_IN];
+  surrogate_begin<T>(dc, s_tc_hdr, cell, w, u14, acc, dt, c, x, nfallback);
+  // the stencil buffers are dead from here on (every thread's accesses ordered before the bulk copies
+  // that reuse them); tiles without a surrogate cell skip the rest
+  tc::fence_async_smem();
+  if (__syncthreads_or(c.kind == 2)) {
+    float y[10];
+    surrogate_tile<TL>(blob, c.kind, x, y, ntimeout, smem, tcx);
+    if (cell) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f) u14[f] = U[f * N + n];
+    }
+    if (c.kind == 2) {
+      Prim<T> w2;
+      cons_to_prim<T, false>(u14, w2);
+      surrogate_end<T>(dc, w2, u14, acc, dt, y, c);
     }
   }
   if (cell) {
-    nactive = kind != 0 ? 1 : 0;
-    lnJh = T(lnJ2[0]);
-    lnJt = T(lnJ2[1]);
-#pragma unroll
-    for (int f = 4; f < 13; ++f) acc[f] += Q[f];
+    nactive = c.kind != 0 ? 1 : 0;
+    lnJh = c.lnJh;
+    lnJt = c.lnJt;
   }
 }
 
@@ -1060,8 +1080,8 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     }
   }
   if (SURR)
-    surrogate_source<TL, T>(dc, blob, cell, w, u14, acc, dt, nactive, nfallback, ntimeout, lnJh, lnJt, smem_raw,
-                            tcx);
+    surrogate_source<TL, T>(dc, blob, cell, w, Uin, N, (size_t)j * nx + i, u14, acc, dt, nactive, nfallback, ntimeout, lnJh,
+                            lnJt, smem_raw, tcx);
   if (cell) {
     const size_t n = (size_t)j * nx + i;
     // RK combine
@@ -1256,16 +1276,14 @@ template <class TL, class T, int STAGE, bool SURR, bool BI = false, bool SP = fa
 __global__ void __launch_bounds__(TL::NT, TL::template minb<T>())
     k_stage(DevCase dc, const T* __restrict__ Uin, const T* Un, T* Uout, const unsigned char* __restrict__ blob) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  TcCtx tcx;
-  tcx.ready = false;
+  TcCtx tcx{};
   if (SURR) {
     // Take the tensor-core resources up front, also in tiles that will not need them: the
     // SM does not start a second CTA of a kernel that uses TMEM until the first has given
     // up its allocation permit, so a lazy allocation would halve the CTAs per SM.
-    tcx.tmem = tc_acquire();
+    tcx.tmem = tc_acquire(blob);
     tcx.phase = 0;
     tcx.wphase = 0;
-    tcx.ready = true;
   }
   stage_tile<TL, T, STAGE, SURR, BI, SP>(dc, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x, Uin, Un, Uout, blob,
                                  smem_raw, dc.cfl, &tcx);
@@ -1307,13 +1325,11 @@ __global__ void __launch_bounds__(TL::NT, TL::template minb<T>())
   __shared__ int s_t, s_slot;
   const int tid = threadIdx.x;
   const int ncases = bt.ncases, total = bt.total_tiles;
-  TcCtx tcx;
-  tcx.ready = false;
+  TcCtx tcx{};
   if (SURR) {
-    tcx.tmem = tc_acquire();   // includes the barrier
+    tcx.tmem = tc_acquire(blob);   // includes the barrier
     tcx.phase = 0;
     tcx.wphase = 0;
-    tcx.ready = true;
   }
   for (int taken = 0; taken < max_tiles; ++taken) {
     if (tid == 0) {

@@ -541,18 +541,21 @@ __global__ void __launch_bounds__(ST::NT, ST::MINB)
 }
 
 // ---- the surrogate kernel of the FP32 + surrogate step through the column sweep ----------
-// The cells k_sweep<..., Q = true> queued (those its screen keeps), 256 at a time, take the
-// fused path's source (surrogate_source: the features, the BF16 tensor-core network inside
-// the training hull, the plain source outside it, the exact tail), then the RK combine, the
-// output and the partials; the last CTA merges its record with the sweep's and publishes
-// the stage.  A persistent grid: the queue's length is known on the device only.
-// The queue of one case (all threads of every CTA of the launch; tcx: the CTA's tensor-core
-// resources, taken once per launch; pub: the CTA that publishes the stage when nothing is
-// queued).
+// The cells k_sweep<..., Q = true> queued (those its screen keeps), 128 at a time per warpgroup,
+// take the fused path's source (the features, the BF16 tensor-core network inside the training
+// hull, the plain source outside it, the exact tail), then the RK combine, the output and the
+// partials; the last CTA merges its record with the sweep's and publishes the stage.  A persistent
+// grid, one CTA per SM with all the network's weights in shared memory: the queue's length is known
+// on the device only.  Its three warpgroups never wait for one another, so the FP64 islands and
+// FP32 work of one run beside the network layers of the others.  (Two CTAs of 256 threads per SM
+// that streamed the weights layer by layer and compacted the surrogate cells of both their halves
+// into one tile took 223 us for the 155,000 kept cells of a 1024 x 256 plume's stage.)
+// The queue of one case (all threads of every CTA of the launch; pub: the CTA that publishes the
+// stage when nothing is queued).  phase: the group's tensor-core barrier phase.
 template <int STAGE>
 __device__ __forceinline__ void queue_case(const DevCase& dc, const float* __restrict__ Uin, const float* Un,
-                                           float* Uout, const unsigned char* __restrict__ blob, double cfl,
-                                           TcCtx* tcx, unsigned char* smem_raw, int pub) {
+                                           float* Uout, double cfl, unsigned char* smem, uint32_t tmem, uint32_t mbar,
+                                           uint32_t& phase, int pub) {
   using T = float;
   using V = float2;
   constexpr int NT = QueueTile::NT, NP = NF / 2;
@@ -577,8 +580,12 @@ __device__ __forceinline__ void queue_case(const DevCase& dc, const float* __res
   for (int f = 0; f < NF; ++f) rmax[f] = T(0);
   T lnJh = T(-INFINITY), lnJt = T(-INFINITY);
   int nactive = 0, nbad = 0, nfallback = 0, ntimeout = 0;
-  for (unsigned base = blockIdx.x * NT; base < count; base += gridDim.x * NT) {   // uniform
-    const unsigned k = base + tid;
+  const int g3 = tid >> 7;
+  const float* hdr = reinterpret_cast<const float*>(smem + mlp::GS_HDR);
+  bool tc_ok = true;
+  // tiles blockIdx.x + gridDim.x * (group + GROUPS m): the groups of all SMs fill evenly
+  for (unsigned tile = blockIdx.x + gridDim.x * (unsigned)g3; tile * 128u < count; tile += gridDim.x * (unsigned)mlp::GROUPS) {
+    const unsigned k = tile * 128u + (tid & 127);
     const bool cell = k < count;
     size_t n = 0;
     T u14[NF], acc[NF];
@@ -596,14 +603,31 @@ __device__ __forceinline__ void queue_case(const DevCase& dc, const float* __res
 #pragma unroll
       for (int f = 0; f < NF; ++f) u14[f] = acc[f] = T(0);
     }
-    int na = 0, nf = 0;
-    T jh = T(-INFINITY), jt = T(-INFINITY);
-    surrogate_source<QueueTile, T>(dc, blob, cell, w, u14, acc, dt, na, nf, ntimeout, jh, jt, smem_raw, tcx);
+    SurrCell<T> c;
+    float x[CT_MLP_IN];
+    int nf = 0;
+    surrogate_begin<T>(dc, hdr, cell, w, u14, acc, dt, c, x, nf);
+    if (mlp::group_any(g3, c.kind == 2)) {
+      float y[10];
+#pragma unroll
+      for (int q = 0; q < CT_MLP_IN; ++q) x[q] = c.kind == 2 ? (x[q] - hdr[mlp::F_XMEAN + q]) * hdr[mlp::F_XISD + q] : 0.0f;
+      if (tc_ok && !mlp::run_group(smem, g3, x, tmem, mbar, phase, y)) {   // a wait gave up: the step reports it
+        tc_ok = false;
+        if ((tid & 127) == 0) ntimeout += 1;
+      }
+      if (c.kind == 2) {
+#pragma unroll
+        for (int q = 0; q < 10; ++q)
+          y[q] = tc_ok ? fminf(fmaxf(y[q] * hdr[mlp::F_YSD + q] + hdr[mlp::F_YMEAN + q], hdr[mlp::F_YMIN + q]), hdr[mlp::F_YMAX + q])
+                       : hdr[mlp::F_YMEAN + q];
+        surrogate_end<T>(dc, w, u14, acc, dt, y, c);
+      }
+    }
     if (cell) {
-      nactive += na;
+      nactive += c.kind != 0 ? 1 : 0;
       nfallback += nf;
-      lnJh = fmaxf(lnJh, jh);
-      lnJt = fmaxf(lnJt, jt);
+      lnJh = fmaxf(lnJh, c.lnJh);
+      lnJt = fmaxf(lnJt, c.lnJt);
       // the sweep's RK combine, output and partials
       T out[NF];
       const V dt2 = p_make(dt, dt);
@@ -711,31 +735,30 @@ __device__ __forceinline__ void queue_case(const DevCase& dc, const float* __res
 }
 
 template <int STAGE>
-__global__ void __launch_bounds__(QueueTile::NT, 2)
+__global__ void __launch_bounds__(QueueTile::NT, 1)
     k_sweep_queue(DevCase dc, const float* __restrict__ Uin, const float* Un, float* Uout,
                   const unsigned char* __restrict__ blob) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ mlp::GroupTc tcs;
   if (dc.hdr->qcount == 0u) {   // nothing queued: publish the sweep's record, take no TMEM
     if (blockIdx.x == 0 && threadIdx.x == 0) publish_stage(dc.hdr, dc.hdr->pre, STAGE, dc.hdr->dt_cur, dc.cfl);
     return;
   }
-  // tensor-core resources up front (a CTA that has given up its allocation permit may not
-  // allocate again)
-  TcCtx tcx;
-  tcx.tmem = tc_acquire();
-  tcx.phase = 0;
-  tcx.wphase = 0;
-  tcx.ready = true;
-  queue_case<STAGE>(dc, Uin, Un, Uout, blob, dc.cfl, &tcx, smem_raw, 0);
-  tc_release(tcx.tmem);
+  const uint32_t tmem = mlp::group_acquire(&tcs);
+  mlp::load_net(smem_raw, blob);
+  const int g = threadIdx.x >> 7;
+  uint32_t phase = 0;
+  queue_case<STAGE>(dc, Uin, Un, Uout, dc.cfl, smem_raw, tmem + 128u * g, tc::smem_addr(&tcs.bar[g]), phase, 0);
+  mlp::group_release(tmem);
 }
 
 // The batched form: the queues of every case of a batch in turn (cases without one skip).
 template <int STAGE>
-__global__ void __launch_bounds__(QueueTile::NT, 2)
+__global__ void __launch_bounds__(QueueTile::NT, 1)
     k_batch_queue(const __grid_constant__ BatchTable bt, const float* __restrict__ Uin, const float* Un, float* Uout,
                   const unsigned char* __restrict__ blob, double cfl) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ mlp::GroupTc tcs;
   // nothing queued in any case: each case's record is published by one CTA, no TMEM taken.
   // (Every CTA reads the counts before any is reset: a count is reset only after all CTAs
   // have passed that case.)
@@ -749,19 +772,18 @@ __global__ void __launch_bounds__(QueueTile::NT, 2)
           publish_stage(bt.cases[k].hdr, bt.cases[k].hdr->pre, STAGE, bt.cases[k].hdr->dt_cur, cfl);
     return;
   }
-  TcCtx tcx;
-  tcx.tmem = tc_acquire();
-  tcx.phase = 0;
-  tcx.wphase = 0;
-  tcx.ready = true;
+  const uint32_t tmem = mlp::group_acquire(&tcs);
+  mlp::load_net(smem_raw, blob);
+  const int g = threadIdx.x >> 7;
+  uint32_t phase = 0;
   for (int k = 0; k < bt.ncases; ++k) {
     if (bt.cases[k].qoff == 0) continue;
     const long long off = bt.state_off[k];
-    queue_case<STAGE>(bt.cases[k], Uin + off, Un ? Un + off : nullptr, Uout + off, blob, cfl, &tcx, smem_raw,
-                      k % (int)gridDim.x);
+    queue_case<STAGE>(bt.cases[k], Uin + off, Un ? Un + off : nullptr, Uout + off, cfl, smem_raw, tmem + 128u * g,
+                      tc::smem_addr(&tcs.bar[g]), phase, k % (int)gridDim.x);
     __syncthreads();
   }
-  tc_release(tcx.tmem);
+  mlp::group_release(tmem);
 }
 
 template <class ST>
