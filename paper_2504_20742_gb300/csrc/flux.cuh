@@ -237,7 +237,7 @@ struct Transport {
 };
 template <class T>
 __device__ __forceinline__ T sutherland(T Tg) {
-  return T(1.716e-5 * (273.15 + 110.4)) * Tg * m_sqrt(Tg * T(1.0 / 273.15)) * T(1.0 / 273.15) / (Tg + T(110.4));
+  return m_div(T(1.716e-5 * (273.15 + 110.4)) * Tg * m_sqrt(Tg * T(1.0 / 273.15)) * T(1.0 / 273.15), Tg + T(110.4));
 }
 template <class T>
 __device__ __forceinline__ Transport<T> transport(T rho, T Tg, T p, T cp, T nu_t) {
@@ -246,7 +246,7 @@ __device__ __forceinline__ Transport<T> transport(T rho, T Tg, T p, T cp, T nu_t
   t.mu_e = mu + rho * nu_t;
   t.lam_e = cp * (mu * T(1.0 / k::PR) + rho * nu_t * T(1.0 / visc::PR_T));
   t.Dp = nu_t * T(1.0 / visc::SC_T);
-  t.Dv = T(visc::DV0 * 101325.0) * m_exp(T(1.94) * m_log(Tg * T(1.0 / 273.15))) / p + t.Dp;
+  t.Dv = m_div(T(visc::DV0 * 101325.0) * m_exp(T(1.94) * m_log(Tg * T(1.0 / 273.15))), p) + t.Dp;
   return t;
 }
 // temperature and c_p of a cell from its primitive vector (moments scaled per kg)

@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include "fastmath.cuh"
+#include "logexp.cuh"
 
 namespace ct {
 
@@ -59,14 +60,18 @@ constexpr double RHOL_OVER_RHOS_CBRT = 1.0293037494292043;   // (1000/917)^(1/3)
 }  // namespace k
 
 // ---- precision-dependent arithmetic ------------------------------------------------------
-// The FP64 path keeps IEEE division (parity with the CPU oracle); the FP32 path uses the
-// fast approximate division (2 ulp), whose error is far below the FP32 state's own rounding.
+// FP32: the fast approximate division (2 ulp), whose error is far below the FP32 state's own
+// rounding.  FP64: logexp.cuh's quotient (2 ulp).
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+__device__ __forceinline__ double fdiv(double a, double b) { return quot_t(a, b); }
 template <class T>
 __device__ __forceinline__ T frcp(T a) { return fdiv(T(1), a); }
+// Quotients of the source terms: IEEE in FP32; in FP64 a multiplication by logexp.cuh's
+// reciprocal (half the FP64 instructions of the division).
+__device__ __forceinline__ float m_div(float a, float b) { return a / b; }
+__device__ __forceinline__ double m_div(double a, double b) { return quot_t(a, b); }
 // Transport arithmetic (primitive recovery, reconstruction, Roe flux): FP64 divisions by
-// the Newton reciprocal of fastmath.cuh (a few ulp); the source terms keep IEEE division.
+// the Newton reciprocal of fastmath.cuh (a few ulp).
 __device__ __forceinline__ float tdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double tdiv(double a, double b) { return a * rcp_nr(b); }
 __device__ __forceinline__ float trcp(float a) { return __fdividef(1.0f, a); }
@@ -76,18 +81,23 @@ __device__ __forceinline__ bool finite_bits(float x) { return (__float_as_uint(x
 __device__ __forceinline__ bool finite_bits(double x) {
   return ((unsigned long long)__double_as_longlong(x) & 0x7ff0000000000000ull) != 0x7ff0000000000000ull;
 }
+// exact conversion to double; normal floats on the integer pipe (conversions run on the FP64 one)
+__device__ __forceinline__ double to_d(double x) { return x; }
+__device__ __forceinline__ double to_d(float x) {
+  return ((__float_as_uint(x) & 0x7fffffffu) - 0x00800000u) < 0x7f000000u ? f2d_bits(x) : double(x);
+}
 // Explicit precision overloads: a templated call must never promote float to double (the
 // FP64 pipe of GB300 is a small fraction of its FP32 rate).
 __device__ __forceinline__ float m_log(float x) { return logf(x); }
-__device__ __forceinline__ double m_log(double x) { return log(x); }
+__device__ __forceinline__ double m_log(double x) { return log_t(x); }
 __device__ __forceinline__ float m_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double m_rsqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float m_exp(float x) { return expf(x); }
-__device__ __forceinline__ double m_exp(double x) { return exp(x); }
+__device__ __forceinline__ double m_exp(double x) { return exp_t(x); }
 __device__ __forceinline__ float m_expm1(float x) { return expm1f(x); }
-__device__ __forceinline__ double m_expm1(double x) { return expm1(x); }
+__device__ __forceinline__ double m_expm1(double x) { return expm1_t(x); }
 __device__ __forceinline__ float m_sqrt(float x) { return sqrtf(x); }
-__device__ __forceinline__ double m_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ double m_sqrt(double x) { return sqrt_t(x); }
 __device__ __forceinline__ float m_cbrt(float x) { return cbrtf(x); }
 __device__ __forceinline__ double m_cbrt(double x) { return cbrt(x); }
 __device__ __forceinline__ float m_floor(float x) { return floorf(x); }
@@ -95,7 +105,7 @@ __device__ __forceinline__ double m_floor(double x) { return floor(x); }
 // Sound speed from c^2 for the CFL time step: the FP32 path takes c^2 rsqrt(c^2) (no IEEE
 // square root); every kernel that computes a time step uses this one form.
 __device__ __forceinline__ float sound_speed(float c2) { return c2 * rsqrtf(c2); }
-__device__ __forceinline__ double sound_speed(double c2) { return sqrt(c2); }
+__device__ __forceinline__ double sound_speed(double c2) { return sqrt_t(c2); }
 __device__ __forceinline__ float m_fabs(float x) { return fabsf(x); }
 __device__ __forceinline__ double m_fabs(double x) { return fabs(x); }
 
@@ -123,15 +133,50 @@ __device__ __forceinline__ R dln_psat_ice(R T) {
 
 // Saturation temperature at vapour pressure pv: Newton, Clausius-Clapeyron start, 6 steps.
 template <class R, bool ICE>
-__device__ __forceinline__ R t_sat(R lnpv) {
+__device__ __forceinline__ R t_sat_start(R lnpv) {
   const R h0 = ICE ? R(k::HLV0 + k::HSL0) : R(k::HLV0);
-  R T = R(1) / (R(1.0 / k::TREF) - R(k::RV) * (lnpv - R(6.415424237852311)) / h0);  // ln 611.2
+  return R(1) / (R(1.0 / k::TREF) - R(k::RV) * (lnpv - R(6.415424237852311)) / h0);  // ln 611.2
+}
+template <class R, bool ICE>
+__device__ __forceinline__ R t_sat(R lnpv) {
+  R T = t_sat_start<R, ICE>(lnpv);
 #pragma unroll
   for (int it = 0; it < 6; ++it) {
     R f = (ICE ? ln_psat_ice(T) : ln_psat_liq(T)) - lnpv;
     R df = ICE ? dln_psat_ice(T) : dln_psat_liq(T);
     T -= f / df;
   }
+  return T;
+}
+// Both curves ln p_sat of Sonntag from ln T and 1/T.
+template <bool ICE>
+__device__ __forceinline__ double ln_psat_of(double T, double lnT, double iT) {
+  return ICE ? fma(-0.49382577, lnT, fma(-6024.5282, iT, fma(T, fma(T, -1.3198825e-5, 1.0613868e-2), 24.7219 + k::LN100)))
+             : fma(2.433502, lnT, fma(-6096.9385, iT, fma(T, fma(T, 1.673952e-5, -2.711193e-2), 16.635794 + k::LN100)));
+}
+// FP64, the same root: four Newton steps in FP32 (to about 1e-5 K, FP32's resolution of ln p),
+// then two in FP64 with the FP32 slope, whose relative error of 1e-7 leaves the first step at
+// 1e-12 K and the second below rounding.  `lnp` evaluates the curve in FP64.  Six FP64 steps took
+// about 370 FP64-pipe instructions, these take 30 (GB300, one such instruction per 64 issue slots).
+template <bool ICE, class F>
+__device__ __forceinline__ double t_sat_newton(double lnpv, const F& lnp) {
+  const float lp = d2f_bits(lnpv);
+  float Tf = t_sat_start<float, ICE>(lp);
+  float slope = 1.0f;
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const float iT = __fdividef(1.0f, Tf), lnT = __logf(Tf);
+    const float f = ICE ? fmaf(-0.49382577f, lnT, fmaf(-6024.5282f, iT, fmaf(Tf, fmaf(Tf, -1.3198825e-5f, 1.0613868e-2f), float(24.7219 + k::LN100))))
+                        : fmaf(2.433502f, lnT, fmaf(-6096.9385f, iT, fmaf(Tf, fmaf(Tf, 1.673952e-5f, -2.711193e-2f), float(16.635794 + k::LN100))));
+    slope = ICE ? fmaf(iT, fmaf(6024.5282f, iT, -0.49382577f), fmaf(Tf, -2.0f * 1.3198825e-5f, 1.0613868e-2f))
+                : fmaf(iT, fmaf(6096.9385f, iT, 2.433502f), fmaf(Tf, 2.0f * 1.673952e-5f, -2.711193e-2f));
+    slope = __fdividef(1.0f, slope);
+    if (it < 3) Tf = fmaf(lp - f, slope, Tf);
+  }
+  const double sl = f2d_bits(slope);
+  double T = f2d_bits(Tf);
+#pragma unroll
+  for (int it = 0; it < 2; ++it) T = fma(lnpv - lnp(T), sl, T);
   return T;
 }
 
@@ -306,16 +351,21 @@ template <class R>
 __device__ __forceinline__ R prop_sigma(const SrcCase& sc, R T) {
   return sc.tables ? tab_prop(tab_of(sc, R(0)), 2, T, false) : sigma_liq(T);
 }
-// T_sat of reading D with the tabulated curve and its derivative (same start and steps)
+// T_sat of reading D with the closed or the tabulated curve (same root in either precision)
 template <class R, bool ICE>
 __device__ __forceinline__ R prop_tsat(const SrcCase& sc, R lnpv) {
-  if (!sc.tables) return t_sat<R, ICE>(lnpv);
-  const R h0 = ICE ? R(k::HLV0 + k::HSL0) : R(k::HLV0);
-  R T = R(1) / (R(1.0 / k::TREF) - R(k::RV) * (lnpv - R(6.415424237852311)) / h0);
-  const R* tab = tab_of(sc, R(0));
+  if constexpr (std::is_same<R, double>::value) {
+    if (sc.tables) return t_sat_newton<ICE>(lnpv, [&](double T) { return tab_prop(sc.tab, ICE ? 1 : 0, T, false); });
+    return t_sat_newton<ICE>(lnpv, [](double T) { return ln_psat_of<ICE>(T, log_t(T), rcp_t(T)); });
+  } else {
+    if (!sc.tables) return t_sat<R, ICE>(lnpv);
+    R T = t_sat_start<R, ICE>(lnpv);
+    const R* tab = tab_of(sc, R(0));
 #pragma unroll
-  for (int it = 0; it < 6; ++it) T -= (tab_prop(tab, ICE ? 1 : 0, T, false) - lnpv) / tab_prop(tab, ICE ? 1 : 0, T, true);
-  return T;
+    for (int it = 0; it < 6; ++it)
+      T -= (tab_prop(tab, ICE ? 1 : 0, T, false) - lnpv) / tab_prop(tab, ICE ? 1 : 0, T, true);
+    return T;
+  }
 }
 
 // Young's growth law, Eq. (16), split as G = cond * D: cond = lambda / den (m/s per K) and
@@ -328,17 +378,19 @@ struct Growth {
 template <class T>
 __device__ __forceinline__ Growth<T> young_growth(T r, T Tg, T Tsat, T lnS, T sig, T rho_d, T h, T lam,
                                                   T lbar, T gam, T cp) {
-  const T Kn = lbar / (T(2) * r);
-  const T ih = T(1) / h;
+  const T Kn = m_div(lbar, T(2) * r);
+  const T ih = m_div(T(1), h);
   const T nu = T(k::RV) * Tsat * ih *
-               (T(k::ALPHA_Y - 0.5) - T((2.0 - k::QC) / (2.0 * k::QC)) * (gam + T(1)) / (T(2) * gam) * cp * Tsat * ih);
+               (T(k::ALPHA_Y - 0.5) - m_div(T((2.0 - k::QC) / (2.0 * k::QC)) * (gam + T(1)), T(2) * gam) * cp * Tsat * ih);
   const T dT = Tsat - Tg;
-  const T dT_lnS = m_fabs(lnS) < T(1e-8) ? T(k::RV) * Tg * Tsat * ih : dT / lnS;
-  const T dT_rc = dT_lnS * T(2) * sig / (rho_d * T(k::RV) * Tg);
-  const T den = rho_d * h * r * (T(1) / (T(1) + T(2 * k::BETA_Y) * Kn) + T(3.78) * (T(1) - nu) * Kn * T(1.0 / k::PR));
+  const T dT_lnS = m_fabs(lnS) < T(1e-8) ? T(k::RV) * Tg * Tsat * ih : m_div(dT, lnS);
+  const T dT_rc = m_div(dT_lnS * T(2) * sig, rho_d * T(k::RV) * Tg);
+  // 1/(1 + 2 beta Kn); FP64: 1 for beta = 0 without the division
+  const T cont = std::is_same<T, double>::value && k::BETA_Y == 0.0 ? T(1) : m_div(T(1), T(1) + T(2 * k::BETA_Y) * Kn);
+  const T den = rho_d * h * r * (cont + T(3.78) * (T(1) - nu) * Kn * T(1.0 / k::PR));
   Growth<T> g;
-  g.cond = lam / den;
-  g.D = dT - dT_rc / r;
+  g.cond = m_div(lam, den);
+  g.D = dT - m_div(dT_rc, r);
   return g;
 }
 
@@ -346,8 +398,8 @@ __device__ __forceinline__ Growth<T> young_growth(T r, T Tg, T Tsat, T lnS, T si
 // saturation curve slope R_v Tsat^2/h per ln p_v, latent heating (h - R_v T)/c_v per unit Y.
 template <class T>
 __device__ __forceinline__ T relax_slope(T Tsat, T Tg, T h, T Yv, T cv) {
-  const T a = T(k::RV) * Tsat * Tsat / h;
-  return m_fabs(a / Yv + (T(1) - a / Tg) * (h - T(k::RV) * Tg) / cv);
+  const T a = m_div(T(k::RV) * Tsat * Tsat, h);
+  return m_fabs(m_div(a, Yv) + m_div((T(1) - m_div(a, Tg)) * (h - T(k::RV) * Tg), cv));
 }
 
 // Expensive part of the source (what the surrogate stands in for): the effective nucleation
@@ -373,7 +425,7 @@ __device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const 
   // growth over the stage: the exponential solution of the linearised exchange
   const T xsum = BI ? dt * (r.xl + r.xh + r.xs) : dt * (r.xl + r.xs);
   if (xsum > T(0)) {
-    const T theta = -m_expm1(-xsum) / xsum;
+    const T theta = m_div(-m_expm1(-xsum), xsum);
     r.Gl *= theta;
     r.Gs *= theta;
     if (BI) r.Gh *= theta;
@@ -392,36 +444,36 @@ __device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const 
       if (aux) aux[9] = double(l10);
     }
     if (pres_l) {
-      rv = m_cbrt(w.ml[3] / w.ml[0]);   // um
+      rv = m_cbrt(m_div(w.ml[3], w.ml[0]));   // um
       const T rvm = rv * T(1e-6);
       T omega;
       if (BI) {   // droplets of homogeneous origin hold no soot
         omega = Js * T(k::FOUR_PI_3) * rvm * rvm * rvm;
       } else {
-        T chi = w.ns / w.ml[0];
+        T chi = m_div(w.ns, w.ml[0]);
         chi = chi > T(1) ? T(1) : chi;
         omega = Js * T(k::FOUR_PI_3) * rvm * rvm * rvm + T(k::K_IMM * k::NS_SITE * 4.0 * k::PI * sc.rp2) * chi;
       }
       if (aux) aux[10] = double(omega);
-      Nf = w.ml[0] * (-m_expm1(-omega * dt) / dt);   // first-order decay over the stage
+      Nf = w.ml[0] * m_div(-m_expm1(-omega * dt), dt);   // first-order decay over the stage
       rf = rv * T(k::RHOL_OVER_RHOS_CBRT);
     }
     if (BI && pres_h) {
-      rvh = m_cbrt(w.mh[3] / w.mh[0]);
+      rvh = m_cbrt(m_div(w.mh[3], w.mh[0]));
       const T rvm = rvh * T(1e-6);
-      T chi = w.ns / w.mh[0];
+      T chi = m_div(w.ns, w.mh[0]);
       chi = chi > T(1) ? T(1) : chi;
       const T omega = Js * T(k::FOUR_PI_3) * rvm * rvm * rvm + T(k::K_IMM * k::NS_SITE * 4.0 * k::PI * sc.rp2) * chi;
-      Nfh = w.mh[0] * (-m_expm1(-omega * dt) / dt);
+      Nfh = w.mh[0] * m_div(-m_expm1(-omega * dt), dt);
       rfh = rvh * T(k::RHOL_OVER_RHOS_CBRT);
     }
   }
 
   // moment sources (per kg, scaled units), Eq. (21)
-  const T jr = r.Jeff / rho;
+  const T jr = m_div(r.Jeff, rho);
   T dml[4], dms[4], dmh[4];
   {
-    const T jrh = BI ? r.Jh / rho : T(0);
+    const T jrh = BI ? m_div(r.Jh, rho) : T(0);
     T rck = T(1), rvk = T(1), rfk = T(1), rvhk = T(1), rfhk = T(1);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -441,8 +493,8 @@ __device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const 
   }
   // limiters on the flux-updated stage state (reading J)
   auto A = [&](int f) { return acc ? U[f] + dt * acc[f] : U[f]; };
-  const T ir = T(1) / rho;
-  const T idt = T(1) / dt;
+  const T ir = m_div(T(1), rho);
+  const T idt = m_div(T(1), dt);
   if (A(8) * ir + dt * dml[3] <= T(0)) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) dml[q] = -(A(5 + q) * ir) * idt;
@@ -515,11 +567,18 @@ __device__ __forceinline__ Sat<T> saturation(const Prim<T>& w, const SrcCase& sc
   populations(w, s.pres_l, s.pres_s);
   s.pres_h = BI && present_h(w);
   // Eq. (1) in FP64: ln S = ln p_v - ln p_sat(T)
-  double pv = double(w.rho) * double(w.Yv) * k::RV * double(w.Tg);
+  const double Td = to_d(w.Tg);
+  double pv = to_d(w.rho) * to_d(w.Yv) * k::RV * Td;
   pv = pv < 1e-30 ? 1e-30 : pv;
   s.lnpv = m_log(pv);
-  s.lnSl = s.lnpv - prop_lnpl<double>(sc, double(w.Tg));
-  s.lnSi = s.lnpv - prop_lnpi<double>(sc, double(w.Tg));
+  if (sc.tables) {
+    s.lnSl = s.lnpv - tab_prop(sc.tab, 0, Td, false);
+    s.lnSi = s.lnpv - tab_prop(sc.tab, 1, Td, false);
+  } else {   // both curves from one logarithm and one reciprocal
+    const double lnT = m_log(Td), iT = rcp_t(Td);
+    s.lnSl = s.lnpv - ln_psat_of<false>(Td, lnT, iT);
+    s.lnSi = s.lnpv - ln_psat_of<true>(Td, lnT, iT);
+  }
   s.active = s.lnSl > 0.0 || s.pres_l || s.pres_s || s.pres_h;
   return s;
 }
@@ -535,15 +594,15 @@ __device__ __forceinline__ Gas<T> gas_props(const Prim<T>& w) {
   const T Tg = w.Tg;
   const T Yg = T(1) - w.Yl - w.Ys;
   const T Ya = Yg - w.Yv;
-  const T iYg = T(1) / Yg;
+  const T iYg = m_div(T(1), Yg);
   Gas<T> g;
   g.cp_g = (Ya * T(k::CPA) + w.Yv * T(k::CPV)) * iYg;
   const T cv_g = (Ya * T(k::CVA) + w.Yv * T(k::CVV)) * iYg;
-  g.gam_g = g.cp_g / cv_g;
+  g.gam_g = m_div(g.cp_g, cv_g);
   const T Rg_g = (Ya * T(k::RA) + w.Yv * T(k::RV)) * iYg;
-  const T mu_g = T(1.716e-5 * (273.15 + 110.4)) * Tg * m_sqrt(Tg * T(1.0 / 273.15)) * T(1.0 / 273.15) / (Tg + T(110.4));
+  const T mu_g = m_div(T(1.716e-5 * (273.15 + 110.4)) * Tg * m_sqrt(Tg * T(1.0 / 273.15)) * T(1.0 / 273.15), Tg + T(110.4));
   g.lam = mu_g * g.cp_g * T(1.0 / k::PR);
-  g.lbar = T(1.5) * mu_g * m_sqrt(Rg_g * Tg) / w.p;
+  g.lbar = m_div(T(1.5) * mu_g * m_sqrt(Rg_g * Tg), w.p);
   g.hfg = T(k::CPV - k::CL) * Tg + T(k::E0V);
   g.hsg = T(k::CPV - k::CS) * Tg + T(k::E0V - k::E0S);
   return g;
@@ -555,13 +614,13 @@ template <class T>
 __device__ __forceinline__ T kantrowitz_phi(const Prim<T>& w, const Gas<T>& g, double rc, double rhov, T Tsat_l) {
   const T Tg = w.Tg;
   const T rcT = T(rc);
-  const T ih = T(1) / g.hfg;
+  const T ih = m_div(T(1), g.hfg);
   const T nu = T(k::RV) * Tsat_l * ih *
-               (T(k::ALPHA_Y - 0.5) - T(0.5) * (g.gam_g + T(1)) / (T(2) * g.gam_g) * g.cp_g * Tsat_l * ih);
-  const T Knc = g.lbar / (T(2) * rcT);
-  const T alpha_c = g.lam / (rcT * (T(1) + T(3.78) * (T(1) - nu) * Knc * T(1.0 / k::PR)));
-  return T(k::QC) * T(rhov) / alpha_c * m_sqrt(T(k::RV) * Tg * T(1.0 / (2.0 * k::PI))) *
-         (g.hfg * g.hfg / (T(k::RV) * Tg * Tg) - g.hfg / Tg);
+               (T(k::ALPHA_Y - 0.5) - m_div(T(0.5) * (g.gam_g + T(1)), T(2) * g.gam_g) * g.cp_g * Tsat_l * ih);
+  const T Knc = m_div(g.lbar, T(2) * rcT);
+  const T alpha_c = m_div(g.lam, rcT * (T(1) + T(3.78) * (T(1) - nu) * Knc * T(1.0 / k::PR)));
+  return m_div(T(k::QC) * T(rhov), alpha_c) * m_sqrt(T(k::RV) * Tg * T(1.0 / (2.0 * k::PI))) *
+         (m_div(g.hfg * g.hfg, T(k::RV) * Tg * Tg) - m_div(g.hfg, Tg));
 }
 
 // Classical nucleation, Eqs. (3), (4), (9), (10), with the soot gate of J_het (reading F):
@@ -576,22 +635,23 @@ __device__ __forceinline__ Cnt cnt_rates(const Prim<T>& w, double lnSl, const Sr
   const T Tg = w.Tg, rho = w.rho;
   Cnt c;
   const T sig = prop_sigma<T>(sc, Tg);
-  const double sigd = double(sig);
-  c.rc = 2.0 * sigd / (k::RHOL * k::RV * double(Tg) * lnSl);
-  const double dGkT = k::FOUR_PI_3 * sigd * c.rc * c.rc / (k::KB * double(Tg));
-  c.rhov = double(rho) * double(w.Yv);
+  const double sigd = to_d(sig), iT = rcp_t(to_d(Tg));
+  c.rc = sigd * iT * m_div(2.0 / (k::RHOL * k::RV), lnSl);
+  const double dGkT = (k::FOUR_PI_3 / k::KB) * iT * sigd * c.rc * c.rc;
+  c.rhov = to_d(rho) * to_d(w.Yv);
   // ln A = ln q_c + 1/2 ln(2 sigma N_A^3 / (pi M^3)) + 2 ln rho_v - ln rho_l
-  const double lnA = 0.5 * m_log(2.0 * sigd) + 0.5 * m_log(k::NA * k::NA * k::NA / (k::PI * k::MW * k::MW * k::MW)) +
-                     2.0 * m_log(c.rhov) - m_log(k::RHOL);
+  constexpr double LN_NA3 = 175.16962154732786;   // ln(N_A^3 / (pi M^3))
+  constexpr double LN_RHOL = 6.907755278982137;       // ln 1000
+  const double lnA = fma(2.0, m_log(c.rhov), fma(0.5, m_log(2.0 * sigd), 0.5 * LN_NA3 - LN_RHOL));
   const double lnJhom = lnA - dGkT;
   const double lnJhet = lnA - k::FTHETA * dGkT;
   c.Jhom = m_exp(lnJhom);
   c.Jsum = c.Jhom;
   c.Jhet = 0.0;
   lnJ2[0] = lnJhom;
-  const double nsv = double(rho) * double(w.ns);
+  const double nsv = to_d(rho) * to_d(w.ns);
   if (sc.n_soot_ref > 0.0 && nsv > 0.0) {
-    const double gate = nsv / sc.n_soot_ref;
+    const double gate = m_div(nsv, sc.n_soot_ref);
     c.Jhet = m_exp(lnJhet) * gate;
     c.Jsum += c.Jhet;
     lnJ2[1] = lnJhet + m_log(gate);
@@ -612,21 +672,21 @@ __device__ __forceinline__ Rates<T> plain_rates(const Prim<T>& w, const Sat<T>& 
   const T lnpv_t = T(st.lnpv);
   const double lnSl = st.lnSl, lnSi = st.lnSi;
 
-  // nucleation, Eqs. (3)-(6), (10); soot-gated heterogeneous rate
+  // the liquid's saturation temperature, once for nucleation and growth (one place, so that the
+  // lanes of a warp that need it for either take it together)
   T Tsat_l = T(0);
-  bool have_tsat_l = false;
+  if (lnSl > 0.0 || st.pres_l || (BI && st.pres_h) || ext) Tsat_l = prop_tsat<T, false>(sc, lnpv_t);
+  // nucleation, Eqs. (3)-(6), (10); soot-gated heterogeneous rate
   if (lnSl > 0.0) {
     const Cnt c = cnt_rates<T>(w, lnSl, sc, lnJ2);
     const double rc = c.rc, rhov = c.rhov, Jhom = c.Jhom, Jhet = c.Jhet, Jsum = c.Jsum;
     // Eq. (5) with alpha_crit from Young's law at r_crit (reading F)
-    Tsat_l = prop_tsat<T, false>(sc, lnpv_t);
-    have_tsat_l = true;
     const T phi = kantrowitz_phi<T>(w, gs, rc, rhov, Tsat_l);
     if (BI) {   // one moment set per mechanism
-      r.Jeff = T(Jhom) / (T(1) + phi);
-      r.Jh = T(Jhet) / (T(1) + phi);
+      r.Jeff = m_div(T(Jhom), T(1) + phi);
+      r.Jh = m_div(T(Jhet), T(1) + phi);
     } else {
-      r.Jeff = T(Jsum) / (T(1) + phi);
+      r.Jeff = m_div(T(Jsum), T(1) + phi);
     }
     r.rc_um = T(rc * 1e6);
     if (aux) { aux[2] = lnJ2[0]; aux[3] = lnJ2[1]; aux[5] = rc; aux[6] = double(phi); }
@@ -641,22 +701,20 @@ __device__ __forceinline__ Rates<T> plain_rates(const Prim<T>& w, const Sat<T>& 
 
   // growth at r20, Eqs. (16), (21) -- G in um/s, relaxation rates of reading J
   if (st.pres_l) {
-    if (!have_tsat_l) Tsat_l = prop_tsat<T, false>(sc, lnpv_t);
-    const T r20 = m_sqrt(w.ml[2] / w.ml[0]) * T(1e-6);
+    const T r20 = m_sqrt(m_div(w.ml[2], w.ml[0])) * T(1e-6);
     const Growth<T> g = young_growth<T>(r20, Tg, Tsat_l, T(lnSl), prop_sigma<T>(sc, Tg), T(k::RHOL), hfg, lam, lbar, gam_g, cp_g);
     r.Gl = g.cond * g.D * T(1e6);
     r.xl = T(4.0 * k::PI * k::RHOL * 1e-12) * w.ml[2] * g.cond * relax_slope(Tsat_l, Tg, hfg, w.Yv, w.cv);
   }
   if (BI && st.pres_h) {
-    if (!have_tsat_l && !st.pres_l) Tsat_l = prop_tsat<T, false>(sc, lnpv_t);
-    const T r20 = m_sqrt(w.mh[2] / w.mh[0]) * T(1e-6);
+    const T r20 = m_sqrt(m_div(w.mh[2], w.mh[0])) * T(1e-6);
     const Growth<T> g = young_growth<T>(r20, Tg, Tsat_l, T(lnSl), prop_sigma<T>(sc, Tg), T(k::RHOL), hfg, lam, lbar, gam_g, cp_g);
     r.Gh = g.cond * g.D * T(1e6);
     r.xh = T(4.0 * k::PI * k::RHOL * 1e-12) * w.mh[2] * g.cond * relax_slope(Tsat_l, Tg, hfg, w.Yv, w.cv);
   }
   if (st.pres_s) {
     const T Tsat_i = prop_tsat<T, true>(sc, lnpv_t);
-    const T r20 = m_sqrt(w.ms[2] / w.ms[0]) * T(1e-6);
+    const T r20 = m_sqrt(m_div(w.ms[2], w.ms[0])) * T(1e-6);
     const Growth<T> g = young_growth<T>(r20, Tg, Tsat_i, T(lnSi), T(k::SIGMA_SV), T(k::RHOS), hsg, lam, lbar, gam_g, cp_g);
     r.Gs = g.cond * g.D * T(1e6);
     r.xs = T(4.0 * k::PI * k::RHOS * 1e-12) * w.ms[2] * g.cond * relax_slope(Tsat_i, Tg, hsg, w.Yv, w.cv);
@@ -666,7 +724,6 @@ __device__ __forceinline__ Rates<T> plain_rates(const Prim<T>& w, const Sat<T>& 
     ext[3] = double(r.Gs);
     ext[4] = double(r.xl);
     ext[5] = double(r.xs);
-    if (!have_tsat_l) Tsat_l = prop_tsat<T, false>(sc, lnpv_t);
     ext[9] = double(Tsat_l - Tg);
   }
   return r;

@@ -52,6 +52,34 @@ __device__ __forceinline__ float2 shfl_down2(float2 v) {
   return make_float2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
 }
 
+// Phase-change source of a cell the screen keeps, added to its flux divergence in the lane's
+// slots (acc: the field pairs, 32 apart).  Out of line, with the cell's values taken from memory
+// here: inlined, its registers made the sweep spill in every row (2.70 -> 2.80 ms for four steps
+// of the kerosene plume 4096 x 1024, which calls it nowhere).  lnJ: ln J_hom and ln J_het, -inf where
+// there is none.  Returns whether the cell is active.
+static __device__ __noinline__ bool sweep_source(const SrcCase& sc, const float* __restrict__ Uin, size_t N, size_t n, float dt,
+                                                 float2* acc, float2* lnJ) {
+  float u14[NF], a[NF], Q[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) u14[f] = Uin[f * N + n];
+#pragma unroll
+  for (int k2 = 0; k2 < NF / 2; ++k2) {
+    const float2 v = acc[32 * k2];
+    a[2 * k2] = v.x;
+    a[2 * k2 + 1] = v.y;
+  }
+  Prim<float> w;
+  cons_to_prim<float, false>(u14, w);
+  double lnJ2[2];
+  if (!phase_source<float, false>(w, u14, a, dt, sc, Q, lnJ2, nullptr)) return false;
+  *lnJ = make_float2(float(lnJ2[0]), float(lnJ2[1]));
+#pragma unroll
+  for (int f = 4; f < 13; ++f) a[f] += Q[f];
+#pragma unroll
+  for (int k2 = 2; k2 < 7; ++k2) acc[32 * k2] = p_make(a[2 * k2], a[2 * k2 + 1]);
+  return true;
+}
+
 // Q (FP32 + surrogate): the cells the screen keeps are not finished here but queued, with
 // their flux divergence, for k_sweep_queue, which runs the surrogate on them; the stage's
 // record then waits in the header (pre) for that kernel to complete and publish it.
@@ -408,6 +436,12 @@ __device__ __forceinline__ void sweep_tile(const DevCase& dc, int bx, int by, in
         }
       } else if (pending) {
         const size_t n = (size_t)j * nx + i;
+        float2 lnJ;
+        if (sweep_source(dc.sc, Uin, N, n, dt, &s_acc[warp][0][lane], &lnJ)) {
+          nactive += 1;
+          lnJh = fmaxf(lnJh, lnJ.x);
+          lnJt = fmaxf(lnJt, lnJ.y);
+        }
         T u14[NF], acc[NF];
 #pragma unroll
         for (int f = 0; f < NF; ++f) u14[f] = Uin[f * N + n];
@@ -416,17 +450,6 @@ __device__ __forceinline__ void sweep_tile(const DevCase& dc, int bx, int by, in
           const V a = s_acc[warp][k2][lane];
           acc[2 * k2] = a.x;
           acc[2 * k2 + 1] = a.y;
-        }
-        Prim<T> w;
-        cons_to_prim<T, false>(u14, w);
-        T Qs[NF];
-        double lnJ2[2];
-        if (phase_source<T, false>(w, u14, acc, dt, dc.sc, Qs, lnJ2, nullptr)) {
-          nactive += 1;
-          lnJh = fmaxf(lnJh, T(lnJ2[0]));
-          lnJt = fmaxf(lnJt, T(lnJ2[1]));
-#pragma unroll
-          for (int f = 4; f < 13; ++f) acc[f] += Qs[f];
         }
         finish(n, u14, acc);
       }
