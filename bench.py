@@ -99,11 +99,10 @@ def _workload(name):
 # Per-cell figures of the fused stage kernel, from one ncu capture each (see profiles/):
 # FP64 arithmetic per cell-stage executed on the plume (mean of the two stages, 527.9 and
 # 602.2 flops on the 16 x 16 two-CTA tile; the kernels skip the exact zeros of the particle
-# moments in air without liquid or ice; the 16 x 14 tile's larger halo adds 0.5 %: 530.5
-# and 605.2), and DRAM bytes per cell per launch (mean of the two stages) by tile shape,
+# moments in air without liquid or ice), and DRAM bytes per cell per launch (mean of the two stages) by tile shape,
 # reported only for a shape counted on the current kernel.
 FP64_FLOPS_PER_CELL_STAGE = 565.1
-FP64_TRAFFIC_PER_CELL_LAUNCH = {7: 452.0, 8: 392.8}    # 16 x 16 and 16 x 14, two CTAs per SM
+FP64_TRAFFIC_PER_CELL_LAUNCH = {7: 452.0}    # 16 x 16, two CTAs per SM
 FP32_TRAFFIC_PER_CELL_LAUNCH = {9: 140.4}    # the column sweep (28 x 64 strips), four CTAs per SM
 SWEEP_SHAPE = 9   # tile shape index of the column-sweep FP32 kernel (k_sweep)
 # the viscous FP64 kernel (same capture recipe, plume with nu_t = 0.5 m^2/s, 16 x 14 tile:

@@ -356,7 +356,8 @@ ct_status ct_step_static(const ct_case *c, int precision, const double *ufac_row
 /* ---- tile shapes and the autotuner (no counterpart in the paper) -----------------------
  * The fused stage kernel is built for several tile shapes (cells per CTA); the state a step
  * produces does not depend on the shape, only the speed does.  Steps of a case use the
- * shape registered for its (geometry, nx, nr, precision), else shape 0 (32 x 8). */
+ * shape registered for its (geometry, nx, nr, precision), else shape 0 (32 x 8), or in plain
+ * CT_FP64 on small grids (up to 20,480 cells) one of the small tiles (8 x 4, 8 x 2). */
 
 /* Number of tile shapes the library is built with. */
 int ct_tile_shape_count(void);
@@ -367,11 +368,12 @@ ct_status ct_tile_shape(int shape, int *tx, int *ty);
 /* CTAs per SM that the registers of shape `shape`'s kernels at `precision` are budgeted for
  * (more CTAs: more resident warps to hide latency, fewer registers per thread); 0 when the
  * shape has no kernels at that precision.  Some shapes carry one precision only: 32 x 8 and
- * 16 x 16 with three FP32 CTAs per SM, 16 x 12 and 16 x 16 with two FP64 CTAs per SM. */
+ * 16 x 16 with three FP32 CTAs per SM, 16 x 12, 16 x 16 and 16 x 15 with two FP64 CTAs per SM. */
 int ct_tile_shape_ctas(int shape, int precision);
 
 /* Register `shape` for cases with this case's geometry, grid and precision (-1: back to the
- * default).  CT_ERR_ARG when the shape's kernel does not fit an SM at that precision. */
+ * default).  CT_ERR_ARG when the shape's kernel does not fit an SM at that precision, or the
+ * grid is too large for it (the small tiles). */
 ct_status ct_set_tile_shape(const ct_case *c, int precision, int shape);
 
 /* Autotuner: time `reps` first-stage launches of every available shape on state U (device,

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(NT_AUX) k_dt(DevCase dc, const T* __restrict__
     }
     dc.partials[(size_t)blockIdx.x * NPART + threadIdx.x] = a;
   }
-  if (!last_block_reduce(dc, fin)) return;
+  if (!last_block_reduce(dc, fin, &red[0][0])) return;
   if (threadIdx.x == 0) dc.hdr->dt_cur = dc.cfl * fin[0];
 }
 
@@ -332,8 +332,10 @@ const StageSet* stage_set_16x16_o3();
 const StageSet* stage_set_32x8_o3();
 const StageSet* stage_set_16x12_d2();
 const StageSet* stage_set_16x16_d2();
-const StageSet* stage_set_16x14_d2();
+const StageSet* stage_set_16x15_d2();
 const StageSet* stage_set_sweep();
+const StageSet* stage_set_8x4();
+const StageSet* stage_set_8x2();
 const StageSet* stage_set(int shape) {
   switch (shape) {
     case 1: return stage_set_16x16();
@@ -343,8 +345,10 @@ const StageSet* stage_set(int shape) {
     case 5: return stage_set_32x8_o3();
     case 6: return stage_set_16x12_d2();
     case 7: return stage_set_16x16_d2();
-    case 8: return stage_set_16x14_d2();
+    case 8: return stage_set_16x15_d2();
     case 9: return stage_set_sweep();
+    case 10: return stage_set_8x4();
+    case 11: return stage_set_8x2();
     default: return stage_set_32x8();
   }
 }
@@ -364,34 +368,49 @@ static int tiles_y(const ct_case* c, int shape) {
   return (case_nr(c) + ty - 1) / ty;
 }
 static int num_blocks(const ct_case* c, int shape) { return tiles_x(c, shape) * tiles_y(c, shape); }
-// partial records and tile rows the workspace holds: enough for every shape
+static size_t cells_of(const ct_case* c) { return (size_t)c->nx * case_nr(c); }
+// a shape this case's grid may use
+static bool shape_serves(int shape, const ct_case* c) { return !stage_set(shape)->small_grid || cells_of(c) <= SMALL_GRID; }
+// partial records and tile rows the workspace holds: enough for every shape the grid may use
 static int max_blocks(const ct_case* c) {
   int m = 0;
-  for (int s = 0; s < NSHAPES; ++s) m = std::max(m, num_blocks(c, s));
+  for (int s = 0; s < NSHAPES; ++s)
+    if (shape_serves(s, c)) m = std::max(m, num_blocks(c, s));
   return m;
 }
 static int max_rows(const ct_case* c) {
   int m = 0;
-  for (int s = 0; s < NSHAPES; ++s) m = std::max(m, tiles_y(c, s));
+  for (int s = 0; s < NSHAPES; ++s)
+    if (shape_serves(s, c)) m = std::max(m, tiles_y(c, s));
   return m;
 }
 
 // Shape chosen per (geometry, grid, precision): set by the autotuner or by the caller,
-// else shape 0.  The state does not depend on the choice; only the speed does.
+// else default_shape.  The state does not depend on the choice; only the speed does.
 static std::mutex g_shape_mu;
 static std::map<std::tuple<int, int, int, int>, int> g_shape;
 static std::tuple<int, int, int, int> shape_key(const ct_case* c, int precision) {
   return std::make_tuple(c->geom, c->nx, case_nr(c), variant_of(c, precision));
 }
+// Without a registered shape: 32 x 8 tiles, or for plain FP64 on grids that leave SMs without one
+// the small tiles: 8 x 2 up to 400 of them (a step of the freezing plume 77 x 29: 251 us with 32 x 8
+// tiles, 115 with 8 x 4, 111 with 8 x 2; 150 x 40: 265, 126, 118), 8 x 4 beyond (256 x 64 cells, 1,024
+// tiles of 8 x 2: 194 against 260).  FP32 keeps 32 x 8, so that its totals, summed in FP32 within a
+// warp, are those of a batch's cases; the autotuner may choose the small tiles there.
+static int default_shape(const ct_case* c, int precision) {
+  if (variant_of(c, precision) != 0 || cells_of(c) > SMALL_GRID) return 0;
+  return num_blocks(c, 11) <= 400 ? 11 : 10;
+}
 static int shape_for(const ct_case* c, int precision) {
   std::lock_guard<std::mutex> lk(g_shape_mu);
   auto it = g_shape.find(shape_key(c, precision));
-  return it == g_shape.end() ? 0 : it->second;
+  return it == g_shape.end() ? default_shape(c, precision) : it->second;
 }
 static bool shape_usable(int shape, int variant, const ct_case* c) {
   if (shape < 0 || shape >= NSHAPES) return false;
   const StageSet* ss = stage_set(shape);
   if (ss->plume_inviscid_only && (c->geom != 1 || c->viscous)) return false;
+  if (!shape_serves(shape, c)) return false;
   return ss->stage[variant][0] != nullptr;
 }
 

@@ -96,18 +96,27 @@ __device__ __forceinline__ double* queue_partials(const DevCase& dc, size_t N) {
 // set for: M32 for the FP32 kernels of tiles up to 320 threads (2: 96 registers; 3: 72
 // registers, more warps to hide latency at the price of spills), else one; M64 for the FP64
 // kernels.
-template <int TX_, int TY_, int M32 = 2, int M64 = 1>
+// NT_ given (ITEMS): that many threads, a multiple of 128, and the slopes handed out as (cell,
+// field pair) items.  Each of an SM's four schedulers has its own FP64 pipe and takes 64 cycles
+// per FP64 instruction of a warp, however few of its lanes are active and whatever the other
+// pipes do (measured: chains of dependent and of independent DFMA alike), so an FP64 phase lasts
+// as long as its busiest scheduler's share: warps in multiples of four, lanes full, work even.
+// SEP: the r faces have buffers of their own, and slopes and fluxes of both directions run as one
+// phase each (small tiles: the length of the chain counts, not shared memory).
+template <int TX_, int TY_, int M32 = 2, int M64 = 1, int NT_ = 0, bool SEP_ = false>
 struct Tile {
   static constexpr int TX = TX_, TY = TY_, HX = TX + 4, HY = TY + 4, NCELL = TX * TY;
-  static constexpr int NFACE = (TX + 1) * TY > TX * (TY + 1) ? (TX + 1) * TY : TX * (TY + 1);
-  static constexpr int NT = (NFACE + 31) / 32 * 32;
+  static constexpr int NFX_ = (TX + 1) * TY, NFR_ = TX * (TY + 1);   // x faces, r faces
+  static constexpr int NFACE = NFX_ > NFR_ ? NFX_ : NFR_;
+  static constexpr bool ITEMS = NT_ != 0, SEP = SEP_;
+  static constexpr int NT = ITEMS ? NT_ : (NFACE + 31) / 32 * 32;
   // The r slopes of rows -1..TY outnumber the threads for the 32-wide tiles; then the threads
   // without a cell take row -1 during the x divergence (see stage_tile).
-  static constexpr bool ROWM1_EARLY = TX * (TY + 2) > NT && NT - NCELL >= TX;
+  static constexpr bool ROWM1_EARLY = !ITEMS && TX * (TY + 2) > NT && NT - NCELL >= TX;
   // Face buffers: left and right reconstructed states; each face's flux overwrites its left
   // state (the thread that read it writes it).  Row -1's r slopes, written during the x
   // divergence while the x fluxes are still read, go to a side buffer of TX faces.
-  static constexpr int NFBUF = 2;
+  static constexpr int NFBUF = SEP ? 4 : 2;
   static constexpr int NSIDE = ROWM1_EARLY ? TX : 0;
   template <class T>
   static constexpr int minb() { return sizeof(T) == 4 ? (NT <= 320 ? M32 : 1) : M64; }
@@ -304,20 +313,35 @@ __device__ __forceinline__ double warp_max_any(double v) {
 __device__ __forceinline__ int slot_kind(int q) { return q == 0 ? 2 : ((q >= 9 && q <= 24) ? 1 : 0); }
 
 // Reduce n partial records (NPART slots each, consecutive) at `base` into out[NPART]
-// (shared memory), in a fixed order: lane-strided over the records, then a warp tree.
-// All threads call this; it ends with a barrier.
-__device__ inline void reduce_records(const double* base, int n, double* out) {
+// (shared memory), in a fixed order: a warp takes every nwarps-th record, a lane per slot, and the
+// warps' results are combined in order.  Sums take one FP64 instruction per record and warp, maxima
+// and minima the integer pipe (a slot per warp with the records over its lanes took five FP64
+// shuffle steps per slot, 64 cycles each: 3,100 cycles for 15 records on four warps, now 600).
+// NaN records count as absent in maxima and minima.  scratch: NPART doubles per warp, shared.  All
+// threads call this; it ends with a barrier.
+__device__ __forceinline__ double fold_slot(int kind, double a, double v) {
+  if (kind == 0) return a + v;
+  const long long ka = order_key(a), kv = order_key(v);
+  const bool nan = (__double_as_longlong(v) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+  return !nan && (kind == 1 ? kv > ka : kv < ka) ? v : a;
+}
+__device__ inline void reduce_records(const double* base, int n, double* out, double* scratch) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
-  for (int q = warp; q < NPART; q += nwarps) {
-    const int kind = slot_kind(q);
-    double acc = kind == 0 ? 0.0 : (kind == 1 ? -INFINITY : INFINITY);
-    for (int b = lane; b < n; b += 32) {
-      const double v = __ldcg(&base[(size_t)b * NPART + q]);
-      acc = kind == 0 ? acc + v : (kind == 1 ? fmax(acc, v) : fmin(acc, v));
-    }
-    acc = kind == 0 ? warp_sum(acc) : (kind == 1 ? warp_max(acc) : warp_min(acc));
-    if (lane == 0) out[q] = acc;
+  const int kind = slot_kind(lane);
+  const double none = kind == 0 ? 0.0 : (kind == 1 ? -INFINITY : INFINITY);
+  if (lane < NPART) {
+    double acc = none;
+#pragma unroll 8
+    for (int b = warp; b < n; b += nwarps) acc = fold_slot(kind, acc, __ldcg(&base[(size_t)b * NPART + lane]));
+    scratch[warp * NPART + lane] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < NPART) {
+    double acc = none;
+    const int m = n < nwarps ? n : nwarps;
+    for (int w = 0; w < m; ++w) acc = fold_slot(kind, acc, scratch[w * NPART + lane]);
+    out[lane] = acc;
   }
   __syncthreads();
 }
@@ -325,7 +349,7 @@ __device__ inline void reduce_records(const double* base, int n, double* out) {
 // Called by all threads after threads 0..NPART-1 wrote this CTA's partial record.  Returns
 // true in the last CTA to arrive (out[] then holds the totals of the dc.nblocks records).
 // One level: for launches of a few hundred CTAs (the time-step kernel).
-__device__ inline bool last_block_reduce(const DevCase& dc, double* out) {
+__device__ inline bool last_block_reduce(const DevCase& dc, double* out, double* scratch) {
   __shared__ unsigned int ticket;
   if (threadIdx.x < NPART) __threadfence();   // the record's writers publish it
   __syncthreads();
@@ -333,7 +357,7 @@ __device__ inline bool last_block_reduce(const DevCase& dc, double* out) {
   __syncthreads();
   if (ticket != (unsigned int)(dc.nblocks - 1)) return false;
   __threadfence();
-  reduce_records(dc.partials, dc.nblocks, out);
+  reduce_records(dc.partials, dc.nblocks, out, scratch);
   if (threadIdx.x == 0) dc.hdr->counter = 0u;
   return true;
 }
@@ -342,8 +366,8 @@ __device__ inline bool last_block_reduce(const DevCase& dc, double* out) {
 // row's records into a row record, and the last row to complete reduces the row records.
 // Both orders are fixed, so the totals are deterministic; no CTA waits for another, and
 // the serial part on the critical path is one row of records instead of all of them.
-// `by`: this tile's row.  Returns true in the CTA that completed the case.
-__device__ inline bool tile_reduce(const DevCase& dc, int by, double* out) {
+// `by`: this tile's row; scratch as reduce_records.  Returns true in the CTA that completed the case.
+__device__ inline bool tile_reduce(const DevCase& dc, int by, double* out, double* scratch) {
   __shared__ unsigned int ticket;
   if (threadIdx.x < NPART) __threadfence();   // the record's writers publish it
   __syncthreads();
@@ -351,7 +375,7 @@ __device__ inline bool tile_reduce(const DevCase& dc, int by, double* out) {
   __syncthreads();
   if (ticket != (unsigned int)(dc.tiles_x - 1)) return false;
   __threadfence();
-  reduce_records(dc.partials + (size_t)by * dc.tiles_x * NPART, dc.tiles_x, out);
+  reduce_records(dc.partials + (size_t)by * dc.tiles_x * NPART, dc.tiles_x, out, scratch);
   if (threadIdx.x < NPART) {
     dc.row_part[(size_t)by * NPART + threadIdx.x] = out[threadIdx.x];
     __threadfence();
@@ -362,7 +386,7 @@ __device__ inline bool tile_reduce(const DevCase& dc, int by, double* out) {
   __syncthreads();
   if (ticket != (unsigned int)(dc.tiles_y - 1)) return false;
   __threadfence();
-  reduce_records(dc.row_part, dc.tiles_y, out);
+  reduce_records(dc.row_part, dc.tiles_y, out, scratch);
   if (threadIdx.x == 0) dc.hdr->counter = 0u;
   return true;
 }
@@ -656,6 +680,9 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   V (*fL2)[NFACE] = reinterpret_cast<V (*)[NFACE]>(smem_raw + sizeof(T) * NFX * HX * HY);  // left states
   V (*fR2)[NFACE] = fL2 + NP;                                       // right states
   V (*fb2)[NFACE] = fL2;                                            // face fluxes
+  // r faces: the same buffers after the x divergence, or their own (SEP)
+  V (*gL2)[NFACE] = TL::SEP ? fR2 + NP : fL2;
+  V (*gR2)[NFACE] = TL::SEP ? fR2 + 2 * NP : fR2;
   // left states of the r faces of row 0 from the early row -1 slopes (32-wide tiles)
   V (*fLm1)[TL::NSIDE > 0 ? TL::NSIDE : 1] =
       reinterpret_cast<V (*)[TL::NSIDE > 0 ? TL::NSIDE : 1]>(fR2 + NP);
@@ -666,6 +693,10 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   };
   const auto fb = [&](int f, int face) -> T {
     const V v = fb2[f >> 1][face];
+    return (f & 1) ? v.y : v.x;
+  };
+  const auto gb = [&](int f, int face) -> T {   // r faces
+    const V v = gL2[f >> 1][face];
     return (f & 1) ? v.y : v.x;
   };
   constexpr bool IS64 = std::is_same<T, double>::value;
@@ -766,37 +797,45 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   const T dt = s_dt;
 
   // phase B1: limited x slopes, once per cell, written as the states of its two faces
-  // (tile-local cell c in [-1, TX]; face f lies between cells f-1 and f)
-  const auto phase_b1 = [&](auto dry_tag) {
+  // (tile-local cell c in [-1, TX]; face f lies between cells f-1 and f): cell p, pairs k_lo .. k_hi - 1
+  constexpr int NSX = (TX + 2) * TY, NSR = TX * (TY + 2);
+  const auto x_slope = [&](int p, int k_lo, int k_hi, auto dry_tag) {
     constexpr bool DRY = decltype(dry_tag)::value;
-    for (int p = tid; p < (TX + 2) * TY; p += NT) {
-      const int c = p % (TX + 2) - 1, hj = p / (TX + 2);
-      const int i = i0 + c, j = j0 + hj;
-      if (i > nx || j >= nr) continue;
+    const int c = p % (TX + 2) - 1, hj = p / (TX + 2);
+    const int i = i0 + c, j = j0 + hj;
+    if (i > nx || j >= nr) return;
 #pragma unroll
-      for (int k2 = 0; k2 < NP; ++k2) {
-        if (DRY && moment_pair(k2)) continue;   // +0 face states, not stored
-        const V am = qs2[k2][hj + 2][c + 1], a0 = qs2[k2][hj + 2][c + 2], a1 = qs2[k2][hj + 2][c + 3];
-        V flo, fhi;
-        vl_faces2(am, a0, a1, flo, fhi);
-        if (c < TX) fL2[k2][hj * (TX + 1) + c + 1] = fhi;
-        if (c >= 0) fR2[k2][hj * (TX + 1) + c] = flo;
-      }
+    for (int k2 = k_lo; k2 < k_hi; ++k2) {
+      if (DRY && moment_pair(k2)) continue;   // +0 face states, not stored
+      const V am = qs2[k2][hj + 2][c + 1], a0 = qs2[k2][hj + 2][c + 2], a1 = qs2[k2][hj + 2][c + 3];
+      V flo, fhi;
+      vl_faces2(am, a0, a1, flo, fhi);
+      if (c < TX) fL2[k2][hj * (TX + 1) + c + 1] = fhi;
+      if (c >= 0) fR2[k2][hj * (TX + 1) + c] = flo;
     }
   };
-  if (dry)
-    phase_b1(std::true_type{});
-  else
-    phase_b1(std::false_type{});
-  __syncthreads();
-
-  // phase B2: x-face Roe fluxes
-  const auto phase_b2 = [&](auto dry_tag) {
+  // limited r slope of tile-local row c in [-1, TY] at column hi -> states of its r faces
+  const auto r_slope = [&](int hi, int c, int k_lo, int k_hi, auto dry_tag) {
     constexpr bool DRY = decltype(dry_tag)::value;
-  for (int p = tid; p < (TX + 1) * TY; p += NT) {
+    const int ii = i0 + hi, jj = j0 + c;
+    if (ii >= nx || jj > nr) return;
+#pragma unroll
+    for (int k2 = k_lo; k2 < k_hi; ++k2) {
+      if (DRY && moment_pair(k2)) continue;   // +0 face states, not stored
+      const V am = qs2[k2][c + 1][hi + 2], a0 = qs2[k2][c + 2][hi + 2], a1 = qs2[k2][c + 3][hi + 2];
+      V flo, fhi;
+      vl_faces2(am, a0, a1, flo, fhi);
+      if (TL::ROWM1_EARLY && c < 0) fLm1[k2][hi] = fhi;
+      else if (c < TY) gL2[k2][(c + 1) * TX + hi] = fhi;
+      if (c >= 0) gR2[k2][c * TX + hi] = flo;
+    }
+  };
+  // Roe flux of x face p, and of r face p (face fy lies between tile rows fy-1 and fy)
+  const auto x_flux = [&](int p, auto dry_tag) {
+    constexpr bool DRY = decltype(dry_tag)::value;
     const int fx = p % (TX + 1), hj = p / (TX + 1);
     const int i = i0 + fx, j = j0 + hj;
-    if (i > nx || j >= nr) continue;
+    if (i > nx || j >= nr) return;
     T qL[NFX], qR[NFX], F[NFX];
 #pragma unroll
     for (int k2 = 0; k2 < NP; ++k2) {
@@ -818,42 +857,90 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     }
 #pragma unroll
     for (int k2 = 0; k2 < NP; ++k2) fb2[k2][p] = p_make(F[2 * k2], F[2 * k2 + 1]);
-  }
   };
-  if (dry)
-    phase_b2(std::true_type{});
-  else
-    phase_b2(std::false_type{});
+  const auto r_flux = [&](int p, auto dry_tag) {
+    constexpr bool DRY = decltype(dry_tag)::value;
+    const int hi = p % TX, fy = p / TX;
+    const int ii = i0 + hi, jj = j0 + fy;
+    if (ii >= nx || jj > nr) return;
+    T qL[NFX], qR[NFX], F[NFX];
+#pragma unroll
+    for (int k2 = 0; k2 < NP; ++k2) {
+      if (DRY && moment_pair(k2)) {
+        qL[2 * k2] = qL[2 * k2 + 1] = qR[2 * k2] = qR[2 * k2 + 1] = T(0);
+        continue;
+      }
+      const V a = (TL::ROWM1_EARLY && p < TX) ? fLm1[k2][p] : gL2[k2][p], b = gR2[k2][p];
+      qL[2 * k2] = a.x;
+      qL[2 * k2 + 1] = a.y;
+      qR[2 * k2] = b.x;
+      qR[2 * k2 + 1] = b.y;
+    }
+    roe_flux<T, 1, NFX, DRY>(qL, qR, F);
+    if (dc.viscous && !(jj == nr && dc.bc_rhi == 1)) {
+      const auto q = [&](int f, int side) -> T { return qs(f, fy + 1 + side, hi + 2); };
+      sub_diffusive_flux<T, NFX>(q, g.idr, g.nu_t, F);
+    }
+#pragma unroll
+    for (int k2 = 0; k2 < NP; ++k2) gL2[k2][p] = p_make(F[2 * k2], F[2 * k2 + 1]);
+  };
+  const auto with_dry = [&](const auto& f) {   // f with the tile's dryness as a compile-time flag
+    if (dry)
+      f(std::true_type{});
+    else
+      f(std::false_type{});
+  };
+  // the slopes of both directions as (cell, pair) items
+  const auto x_items = [&](auto t) {
+    for (int p = tid; p < NSX * NP; p += NT) x_slope(p % NSX, p / NSX, p / NSX + 1, t);
+  };
+  const auto r_items = [&](auto t) {
+    for (int p = tid; p < NSR * NP; p += NT) r_slope(p % TX, p % NSR / TX - 1, p / NSR, p / NSR + 1, t);
+  };
+  if constexpr (TL::SEP) {
+    with_dry([&](auto t) {
+      x_items(t);
+      if (dc.geom == 1) r_items(t);
+    });
+    __syncthreads();
+    // x faces on the first warps, r faces on the next ones
+    constexpr int XW = (TL::NFX_ + 31) / 32 * 32;
+    with_dry([&](auto t) {
+      for (int p = tid; p < XW + TL::NFR_; p += NT) {
+        if (p < TL::NFX_)
+          x_flux(p, t);
+        else if (p >= XW && dc.geom == 1)
+          r_flux(p - XW, t);
+      }
+    });
+  } else {
+    with_dry([&](auto t) {
+      if constexpr (TL::ITEMS) {
+        x_items(t);
+      } else {
+        for (int p = tid; p < NSX; p += NT) x_slope(p, 0, NP, t);
+      }
+    });
+    __syncthreads();
+    // phase B2: x-face Roe fluxes
+    with_dry([&](auto t) {
+      for (int p = tid; p < TL::NFX_; p += NT) x_flux(p, t);
+    });
+  }
   __syncthreads();
 
   const int ci = tid % TX, cj = tid / TX;
   const int i = i0 + ci, j = j0 + cj;
   const bool cell = tid < NCELL && i < nx && j < nr;
-  // limited r slope of tile-local row c in [-1, TY] at column hi -> states of its r faces
-  const auto r_slope = [&](int hi, int c, auto dry_tag) {
-    constexpr bool DRY = decltype(dry_tag)::value;
-    const int ii = i0 + hi, jj = j0 + c;
-    if (ii >= nx || jj > nr) return;
-#pragma unroll
-    for (int k2 = 0; k2 < NP; ++k2) {
-      if (DRY && moment_pair(k2)) continue;   // +0 face states, not stored
-      const V am = qs2[k2][c + 1][hi + 2], a0 = qs2[k2][c + 2][hi + 2], a1 = qs2[k2][c + 3][hi + 2];
-      V flo, fhi;
-      vl_faces2(am, a0, a1, flo, fhi);
-      if (TL::ROWM1_EARLY && c < 0) fLm1[k2][hi] = fhi;
-      else if (c < TY) fL2[k2][(c + 1) * TX + hi] = fhi;
-      if (c >= 0) fR2[k2][c * TX + hi] = flo;
-    }
-  };
   // The r slopes of rows -1..TY outnumber the threads for the 32-wide tiles; the threads
   // without a cell take row -1 during the x divergence (the x face states are dead by then),
   // so that phase D1 is a single round.
   constexpr bool ROWM1_EARLY = TL::ROWM1_EARLY;
   T acc[NFX];
   // water carried by a face flux: vapour, liquid (both sets) and ice
-  const auto water_flux = [&](int f) -> T {
-    const T l3 = BI ? fb(8, f) + fb(17, f) : fb(8, f);
-    return fb(4, f) + T(k::YL3) * l3 + T(k::YS3) * fb(12, f);
+  const auto water_flux = [&](const auto& b, int f) -> T {
+    const T l3 = BI ? b(8, f) + b(17, f) : b(8, f);
+    return b(4, f) + T(k::YL3) * l3 + T(k::YS3) * b(12, f);
   };
   T bm = T(0), bw = T(0), be = T(0);   // boundary inflow rates of this cell's faces
   T area_w = T(0), area_e = T(0), vol = T(0);
@@ -907,64 +994,33 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     }
     if (i == 0) {
       bm += area_w * fb(0, w);
-      bw += area_w * water_flux(w);
+      bw += area_w * water_flux(fb, w);
       be += area_w * fb(3, w);
     }
     if (i == nx - 1) {
       bm -= area_e * fb(0, e);
-      bw -= area_e * water_flux(e);
+      bw -= area_e * water_flux(fb, e);
       be -= area_e * fb(3, e);
     }
   }
 
-  if (dc.geom == 1) {
-    if (ROWM1_EARLY && tid >= NCELL && tid - NCELL < TX) {
-      if (dry)
-        r_slope(tid - NCELL, -1, std::true_type{});
-      else
-        r_slope(tid - NCELL, -1, std::false_type{});
-    }
+  if (!TL::SEP && dc.geom == 1) {
+    if (ROWM1_EARLY && tid >= NCELL && tid - NCELL < TX)
+      with_dry([&](auto t) { r_slope(tid - NCELL, -1, 0, NP, t); });
     __syncthreads();
     // phase D1: limited r slopes (tile-local row c in [-1, TY]) -> states of the r faces
-    if (dry) {
-      for (int p = tid + (ROWM1_EARLY ? TX : 0); p < TX * (TY + 2); p += NT) r_slope(p % TX, p / TX - 1, std::true_type{});
-    } else {
-      for (int p = tid + (ROWM1_EARLY ? TX : 0); p < TX * (TY + 2); p += NT) r_slope(p % TX, p / TX - 1, std::false_type{});
-    }
+    with_dry([&](auto t) {
+      if constexpr (TL::ITEMS) {
+        r_items(t);
+      } else {
+        for (int p = tid + (ROWM1_EARLY ? TX : 0); p < NSR; p += NT) r_slope(p % TX, p / TX - 1, 0, NP, t);
+      }
+    });
     __syncthreads();
-    // phase D2: r-face Roe fluxes (face fy lies between tile rows fy-1 and fy)
-    const auto phase_d2 = [&](auto dry_tag) {
-      constexpr bool DRY = decltype(dry_tag)::value;
-    for (int p = tid; p < TX * (TY + 1); p += NT) {
-      const int hi = p % TX, fy = p / TX;
-      const int ii = i0 + hi, jj = j0 + fy;
-      if (ii >= nx || jj > nr) continue;
-      T qL[NFX], qR[NFX], F[NFX];
-#pragma unroll
-      for (int k2 = 0; k2 < NP; ++k2) {
-        if (DRY && moment_pair(k2)) {
-          qL[2 * k2] = qL[2 * k2 + 1] = qR[2 * k2] = qR[2 * k2 + 1] = T(0);
-          continue;
-        }
-        const V a = (TL::ROWM1_EARLY && p < TX) ? fLm1[k2][p] : fL2[k2][p], b = fR2[k2][p];
-        qL[2 * k2] = a.x;
-        qL[2 * k2 + 1] = a.y;
-        qR[2 * k2] = b.x;
-        qR[2 * k2 + 1] = b.y;
-      }
-      roe_flux<T, 1, NFX, DRY>(qL, qR, F);
-      if (dc.viscous && !(jj == nr && dc.bc_rhi == 1)) {
-        const auto q = [&](int f, int side) -> T { return qs(f, fy + 1 + side, hi + 2); };
-        sub_diffusive_flux<T, NFX>(q, g.idr, g.nu_t, F);
-      }
-#pragma unroll
-      for (int k2 = 0; k2 < NP; ++k2) fb2[k2][p] = p_make(F[2 * k2], F[2 * k2 + 1]);
-    }
-    };
-    if (dry)
-      phase_d2(std::true_type{});
-    else
-      phase_d2(std::false_type{});
+    // phase D2: r-face Roe fluxes
+    with_dry([&](auto t) {
+      for (int p = tid; p < TL::NFR_; p += NT) r_flux(p, t);
+    });
     __syncthreads();
   }
 
@@ -1021,8 +1077,8 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
       const bool wall_s = wall && j == dc.jw, wall_n = wall && j == dc.jw - 1;
       if constexpr (IS64) {
         const int fs = cj * TX + ci, fn = (cj + 1) * TX + ci;
-        const auto Fs = [&](int f) -> T { return wall_s ? (f == 2 ? w.p : T(0)) : fb(f, fs); };
-        const auto Fn = [&](int f) -> T { return wall_n ? (f == 2 ? w.p : T(0)) : fb(f, fn); };
+        const auto Fs = [&](int f) -> T { return wall_s ? (f == 2 ? w.p : T(0)) : gb(f, fs); };
+        const auto Fn = [&](int f) -> T { return wall_n ? (f == 2 ? w.p : T(0)) : gb(f, fn); };
 #pragma unroll
         for (int f = 0; f < NFX; ++f)
           if (!is_moment(f)) acc[f] = acc[f] + fma(cs, Fs(f), -cn * Fn(f));
@@ -1035,7 +1091,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
         const V cs2 = p_make(cs, cs), ncn2 = p_make(-cn, -cn);
 #pragma unroll
         for (int k2 = 0; k2 < NP; ++k2) {
-          V Fs = fb2[k2][cj * TX + ci], Fn = fb2[k2][(cj + 1) * TX + ci];
+          V Fs = gL2[k2][cj * TX + ci], Fn = gL2[k2][(cj + 1) * TX + ci];
           if (wall_n) Fn = p_make(k2 == 1 ? w.p : T(0), T(0));
           if (wall_s) Fs = p_make(k2 == 1 ? w.p : T(0), T(0));
           const V a = p_add(p_make(acc[2 * k2], acc[2 * k2 + 1]), p_fma(cs2, Fs, p_mul(ncn2, Fn)));
@@ -1052,9 +1108,9 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
       if (j == nr - 1) {
         const T An = T(nr) * g.dr * g.dx;
         const int e = (cj + 1) * TX + ci;
-        bm -= An * fb(0, e);
-        bw -= An * water_flux(e);
-        be -= An * fb(3, e);
+        bm -= An * gb(0, e);
+        bw -= An * water_flux(gb, e);
+        be -= An * gb(3, e);
       }
     } else {
       acc[1] += w.p * tdiv(area_e - area_w, vol);
@@ -1265,7 +1321,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     if (STAGE == 2 && tid >= 9 && tid < 9 + NF) acc2 *= trcp(dt);
     dc.partials[(size_t)tile * NPART + tid] = double(acc2);
   }
-  if (!tile_reduce(dc, by, fin)) return;
+  if (!tile_reduce(dc, by, fin, reinterpret_cast<double*>(smem_raw))) return;   // the stencil buffers are dead
   if (tid == 0) publish_stage(dc.hdr, fin, STAGE, dtd, cfl);
 }
 
@@ -1379,7 +1435,12 @@ struct StageSet {
   const void* queue[2];             // FP32 + surrogate: the kernel after each stage kernel (or null)
   const void* batch_queue[2];       // the same after each batched stage kernel
   size_t queue_smem;                // their dynamic shared memory
+  bool small_grid;                  // for grids of at most SMALL_GRID cells only
 };
+// Largest grid the small tiles serve, in cells.  A step of the freezing plume in FP64 on GB300, 32 x 8
+// tiles / 8 x 4 tiles: 300 x 80 cells 268 / 181 us, a condensing plume 256 x 64 277 / 194 us; on
+// 400 x 100 cells, which give every SM a 32 x 8 tile, 263 / 264 and 280 / 376 us.
+constexpr size_t SMALL_GRID = 20480;
 constexpr size_t SMEM_LIMIT = 227 * 1024 - 4096;   // opt-in limit minus the static shared memory
 
 template <class TL>
@@ -1468,10 +1529,24 @@ StageSet make_stage_set_fp64() {
   return s;
 }
 
+// Plain FP64 and FP32 kernels (variants 0 and 1) of a small tile, for grids that would leave most SMs
+// without one of the larger tiles.
+template <class TL>
+StageSet make_stage_set_small() {
+  StageSet s = make_stage_set_fp64<TL>();
+  s.smem[1] = TL::template smem<float>();
+  s.minb[1] = TL::template minb<float>();
+  s.stage[1][0] = (const void*)k_stage<TL, float, 1, false>;
+  s.stage[1][1] = (const void*)k_stage<TL, float, 2, false>;
+  s.small_grid = true;
+  return s;
+}
+
 // the tile shapes the library is built with (one translation unit each)
-constexpr int NSHAPES = 10;
-// 0: 32x8 (default), 1: 16x16, 2: 32x16, 3: 64x8, 4: 16x16 and 5: 32x8 with three FP32 CTAs
-// per SM, 6: 16x12, 7: 16x16 and 8: 16x14 with two FP64 CTAs per SM
+constexpr int NSHAPES = 12;
+// 0: 32x8, 1: 16x16, 2: 32x16, 3: 64x8, 4: 16x16 and 5: 32x8 with three FP32 CTAs per SM, 6: 16x12,
+// 7: 16x16 and 8: 16x15 with two FP64 CTAs per SM, 9: the column sweep, 10: 8x4 and 11: 8x2 for
+// small grids
 const StageSet* stage_set(int shape);
 
 }  // namespace ct

@@ -507,7 +507,7 @@ __device__ __forceinline__ void sweep_tile(const DevCase& dc, int bx, int by, in
     }
     dc.partials[(size_t)tile * NPART + q] = a;
   }
-  if (!tile_reduce(dc, by, fin)) return;
+  if (!tile_reduce(dc, by, fin, &red[0][0])) return;
   if (threadIdx.x == 0) {
     if (Q) {
       for (int q = 0; q < NPART; ++q) dc.hdr->pre[q] = fin[q];
@@ -742,7 +742,7 @@ __device__ __forceinline__ void queue_case(const DevCase& dc, const float* __res
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
   __threadfence();
-  reduce_records(queue_partials(dc, N), gridDim.x, fin);
+  reduce_records(queue_partials(dc, N), gridDim.x, fin, &red[0][0]);
   if (tid == 0) {
     WsHeader* h = dc.hdr;
     double m[NPART];
