@@ -33,10 +33,12 @@ __device__ __forceinline__ double f2d_bits(float x) {
   const unsigned h = (u & 0x80000000u) | ((a >> 3) + 0x38000000u);
   return __hiloint2double((int)(a >= 0x00800000u ? h : 0u), (int)(a >= 0x00800000u ? u << 29 : 0u));
 }
-// x / 2 on the integer pipe, for zero and for normal x with a normal half
+// x / 2 on the integer pipe: exact for normal x with a normal half; zero, subnormal, infinite and
+// NaN values are returned as they are
 __device__ __forceinline__ double half_bits(double x) {
   const int h = __double2hiint(x);
-  return __hiloint2double((h & 0x7ff00000) ? h - 0x00100000 : h, __double2loint(x));
+  const unsigned e = (unsigned)h & 0x7ff00000u;
+  return __hiloint2double(e - 0x00100000u < 0x7fe00000u ? h - 0x00100000 : h, __double2loint(x));
 }
 
 // CUDA's functions for the other arguments, out of line: their code (some 150 instructions each) is

@@ -275,17 +275,62 @@ __device__ __forceinline__ void cons_to_prim_impl(const T* U, Prim<T>& w) {
   w.p = rn_mul(rn_mul(rho, w.Rg), w.Tg);
   w.c2 = rn_mul(rn_mul(rn_fma(w.Rg, icv, T(1)), w.p), ir);
 }
-// FP64 takes the shorter form where the moments are zero (the FP64 pipe is the bottleneck
-// of the FP64 kernels); FP32 always the full one.
+// FP64: the mixture's constants as differences from dry air's, one operation per constituent, and
+// halves on the integer pipe (the FP64 pipe bounds the FP64 kernels); the same bits with and
+// without ZERO as above.
+template <bool BI, bool ZERO>
+__device__ __forceinline__ void cons_to_prim64(const double* U, Prim<double>& w) {
+  const double rho = U[0];
+  double rcv = fma(U[4], k::CVV - k::CVA, __dmul_rn(rho, k::CVA));
+  if constexpr (!ZERO) {
+    const double rYl = __dmul_rn(k::YL3, BI ? __dadd_rn(U[8], U[17]) : U[8]), rYs = __dmul_rn(k::YS3, U[12]);
+    rcv = fma(rYs, k::CS - k::CVA, fma(rYl, k::CL - k::CVA, rcv));
+  }
+  const double X = rcp_nr(__dmul_rn(rho, rcv));
+  const double ir = __dmul_rn(rcv, X);
+  w.rho = rho;
+  w.u = __dmul_rn(U[1], ir);
+  w.v = __dmul_rn(U[2], ir);
+  w.Yv = __dmul_rn(U[4], ir);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    w.ml[q] = ZERO ? U[5 + q] : __dmul_rn(U[5 + q], ir);
+    w.ms[q] = ZERO ? U[9 + q] : __dmul_rn(U[9 + q], ir);
+  }
+  w.ns = __dmul_rn(U[13], ir);
+  if constexpr (BI) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w.mh[q] = ZERO ? U[14 + q] : __dmul_rn(U[14 + q], ir);
+    w.Yl = ZERO ? w.ml[3] : __dmul_rn(k::YL3, __dadd_rn(w.ml[3], w.mh[3]));
+  } else {
+    w.Yl = ZERO ? w.ml[3] : __dmul_rn(k::YL3, w.ml[3]);
+  }
+  w.Ys = ZERO ? w.ms[3] : __dmul_rn(k::YS3, w.ms[3]);
+  const double ke = half_bits(fma(w.u, w.u, __dmul_rn(w.v, w.v)));
+  double th = fma(-w.Yv, k::E0V, fma(U[3], ir, -ke));   // c_v T
+  w.Rg = fma(w.Yv, k::RV - k::RA, k::RA);
+  if constexpr (!ZERO) {
+    th = fma(-w.Ys, k::E0S, th);
+    w.Rg = fma(-k::RA, __dadd_rn(w.Yl, w.Ys), w.Rg);
+  }
+  w.cv = __dmul_rn(rcv, ir);
+  const double icv = __dmul_rn(__dmul_rn(rho, rho), X);
+  w.Tg = __dmul_rn(th, icv);
+  const double s = __dmul_rn(w.Rg, w.Tg);
+  w.p = __dmul_rn(rho, s);
+  w.c2 = __dmul_rn(fma(w.Rg, icv, 1.0), s);
+}
+// FP32 always takes the full form.
 template <class T, bool BI = false>
 __device__ __forceinline__ void cons_to_prim(const T* U, Prim<T>& w) {
   if constexpr (std::is_same<T, double>::value) {
-    if (moments_zero<nf_of<BI>()>([&](int f) { return U[f]; })) {
-      cons_to_prim_impl<T, BI, true>(U, w);
-      return;
-    }
+    if (moments_zero<nf_of<BI>()>([&](int f) { return U[f]; }))
+      cons_to_prim64<BI, true>(U, w);
+    else
+      cons_to_prim64<BI, false>(U, w);
+  } else {
+    cons_to_prim_impl<T, BI, false>(U, w);
   }
-  cons_to_prim_impl<T, BI, false>(U, w);
 }
 
 // Conserved state from (p, T, u, v, Y_v, scaled moments, soot per kg).

@@ -637,6 +637,10 @@ __device__ __forceinline__ void surrogate_source(const DevCase& dc, const unsign
 }
 
 
+// x / 2 (FP64 on the integer pipe)
+__device__ __forceinline__ double half_of(double x) { return half_bits(x); }
+__device__ __forceinline__ float half_of(float x) { return 0.5f * x; }
+
 // planes of stored primitive variables per state: the stencil's fields, T and c_v
 constexpr int NPLANE = NF + 2;
 
@@ -718,7 +722,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   // columns, once per row and column with the expressions the cells would evaluate
   // themselves (the same bits), published by phase A's barrier.  The FP32 kernels keep the
   // per-cell form: their shared memory is the tighter budget.
-  __shared__ T s_row[IS64 ? TY : 1][5];
+  __shared__ T s_row[IS64 ? TY : 1][6];
   __shared__ bool s_wall[IS64 ? TX : 1];
   if (IS64 && dc.geom == 1) {
     for (int r = tid; r < TY; r += NT) {
@@ -730,6 +734,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
       s_row[r][2] = T(j + 1) * ijh * g.idr;
       s_row[r][3] = area;
       s_row[r][4] = area * g.dx;
+      s_row[r][5] = ijh * g.idr;
     }
     for (int c = tid; c < TX; c += NT) s_wall[c] = g.wall_len > T(0) && (T(i0 + c) + T(0.5)) * g.dx < g.wall_len;
   }
@@ -1081,11 +1086,11 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
         const auto Fn = [&](int f) -> T { return wall_n ? (f == 2 ? w.p : T(0)) : gb(f, fn); };
 #pragma unroll
         for (int f = 0; f < NFX; ++f)
-          if (!is_moment(f)) acc[f] = acc[f] + fma(cs, Fs(f), -cn * Fn(f));
+          if (!is_moment(f)) acc[f] = fma(cs, Fs(f), fma(-cn, Fn(f), acc[f]));
         if (!(moments_zero<NFX>(Fs) && moments_zero<NFX>(Fn))) {   // as in the x divergence
 #pragma unroll
           for (int f = 0; f < NFX; ++f)
-            if (is_moment(f)) acc[f] = acc[f] + fma(cs, Fs(f), -cn * Fn(f));
+            if (is_moment(f)) acc[f] = fma(cs, Fs(f), fma(-cn, Fn(f), acc[f]));
         }
       } else {
         const V cs2 = p_make(cs, cs), ncn2 = p_make(-cn, -cn);
@@ -1099,7 +1104,8 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
           acc[2 * k2 + 1] = a.y;
         }
       }
-      acc[2] += w.p * ijh * g.idr;
+      if constexpr (IS64) acc[2] = fma(w.p, s_row[cj][5], acc[2]);
+      else acc[2] += w.p * ijh * g.idr;
       if (dc.viscous) {   // radial component of the vector Laplacian: -mu_e v / r^2
         T mu_e;
         viscous_rate<T>(w, g.nu_t, T(0), mu_e);
@@ -1192,7 +1198,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
       for (int f = 0; f < NFX; ++f) {
         if (is_moment(f)) continue;
         const T un = Un[f * N + n];
-        out[f] = fma(T(0.5), un, T(0.5) * fma(dt, acc[f], u14[f]));
+        out[f] = fma(T(0.5), un, half_of(fma(dt, acc[f], u14[f])));
         if (f < NF) rmax[f] = m_fabs(out[f] - un);   // divided by dt once per CTA
       }
       if (mz) {
@@ -1207,7 +1213,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
         for (int f = 0; f < NFX; ++f) {
           if (!is_moment(f)) continue;
           const T un = Un[f * N + n];
-          out[f] = fma(T(0.5), un, T(0.5) * fma(dt, acc[f], u14[f]));
+          out[f] = fma(T(0.5), un, half_of(fma(dt, acc[f], u14[f])));
           const T rf = m_fabs(out[f] - un);
           if (f < NF) {
             rmax[f] = rf;

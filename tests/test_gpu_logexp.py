@@ -106,9 +106,9 @@ def test_conversion_and_halving_are_exact(lib):
     x = np.concatenate([g.integers(0, 1 << 32, 4096, dtype=np.uint32).view(np.float32).astype(np.float64), [0.0, -0.0, np.inf, 1e-45, 1.0]])
     got, ref = lib(5, x)
     assert np.array_equal(got, ref, equal_nan=True)
-    x = np.concatenate([np.exp(-600 + 1200 * g.random(4096)), [0.0, -3.0]])
+    x = np.concatenate([np.exp(-600 + 1200 * g.random(4096)), [0.0, -3.0, np.inf, -np.inf, np.nan]])
     got, ref = lib(6, x)
-    assert np.array_equal(got, ref)
+    assert np.array_equal(got, ref, equal_nan=True)
 
 
 # The root's condition: rounding of ln p (a few ulp of its largest term, 30 to 100: 1e-14) over the
