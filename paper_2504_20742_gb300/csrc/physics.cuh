@@ -447,6 +447,11 @@ __device__ __forceinline__ T relax_slope(T Tsat, T Tg, T h, T Yv, T cv) {
   return m_fabs(m_div(a, Yv) + m_div((T(1) - m_div(a, Tg)) * (h - T(k::RV) * Tg), cv));
 }
 
+// a * b, in FP64 with a rounding of its own (never one half of a fused multiply-add): results that
+// one warp may hand to another through shared memory have the same bits there as in registers
+__device__ __forceinline__ double own_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float own_mul(float a, float b) { return a * b; }
+
 // Expensive part of the source (what the surrogate stands in for): the effective nucleation
 // rate J/(1+phi) (m^-3 s^-1) and critical radius (um), the raw growth rates G(r20) (um/s) and
 // the relaxation rates 1/tau of the linearised vapour exchange (1/s) of both phases.
@@ -456,29 +461,18 @@ struct Rates {
   T Jh, Gh, xh;   // bimodal: heterogeneous nucleation, growth and relaxation of the second set
 };
 
-// Cheap part of the source, shared by the plain and the surrogate paths: relaxation
-// limiter, freezing, moment assembly (Eq. 21), vapour sink (Eqs. 18, 25) and the
-// flux-aware limiters of reading J.  U: conserved stage input of the cell; acc (may be
-// null): its flux-only residual, so that the limiters act on A = U + dt acc.  BI: the
-// bimodal liquid, whose second set (fields 14..17) takes the heterogeneous nucleation
-// r.Jh, grows at r.Gh and alone freezes by immersion.
-template <class T, bool BI = false>
-__device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const T* acc, T dt, const SrcCase& sc,
-                                            bool pres_l, bool pres_s, double lnSl, double lnSi, Rates<T> r, T* Q,
-                                            double* aux, bool pres_h = false) {
-  const T Tg = w.Tg, rho = w.rho;
-  // growth over the stage: the exponential solution of the linearised exchange
-  const T xsum = BI ? dt * (r.xl + r.xh + r.xs) : dt * (r.xl + r.xs);
-  if (xsum > T(0)) {
-    const T theta = m_div(-m_expm1(-xsum), xsum);
-    r.Gl *= theta;
-    r.Gs *= theta;
-    if (BI) r.Gh *= theta;
-  }
-  if (aux) { aux[7] = double(r.Gl) * 1e-6; aux[8] = double(r.Gs) * 1e-6; }
-
-  // freezing, Eqs. (12)-(15) (reading H); with the bimodal liquid only droplets of
-  // heterogeneous origin carry a soot particle for immersion freezing
+// Freezing of the liquid populations, Eqs. (12)-(15) (reading H): droplets frozen per kg and second,
+// their volume radius and that of the ice they become (um); the second set's with the bimodal liquid.
+template <class T>
+struct Freezing {
+  T Nf, rv, rf, Nfh, rvh, rfh;
+};
+template <class T, bool BI>
+__device__ __forceinline__ Freezing<T> freezing_rates(const Prim<T>& w, T dt, const SrcCase& sc, bool pres_l, bool pres_h,
+                                                      double lnSl, double lnSi, double* aux) {
+  const T Tg = w.Tg;
+  // with the bimodal liquid only droplets of heterogeneous origin carry a soot particle for
+  // immersion freezing
   T Nf = T(0), rv = T(0), rf = T(0), Nfh = T(0), rvh = T(0), rfh = T(0);
   if (sc.freezing && (pres_l || (BI && pres_h)) && Tg < T(k::TREF)) {
     const T daw = T(1) - T(m_exp(lnSl - lnSi));   // 1 - p_sat,i / p_sat,l
@@ -500,7 +494,7 @@ __device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const 
         omega = Js * T(k::FOUR_PI_3) * rvm * rvm * rvm + T(k::K_IMM * k::NS_SITE * 4.0 * k::PI * sc.rp2) * chi;
       }
       if (aux) aux[10] = double(omega);
-      Nf = w.ml[0] * m_div(-m_expm1(-omega * dt), dt);   // first-order decay over the stage
+      Nf = own_mul(w.ml[0], m_div(-m_expm1(-omega * dt), dt));   // first-order decay over the stage
       rf = rv * T(k::RHOL_OVER_RHOS_CBRT);
     }
     if (BI && pres_h) {
@@ -513,7 +507,30 @@ __device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const 
       rfh = rvh * T(k::RHOL_OVER_RHOS_CBRT);
     }
   }
+  return {Nf, rv, rf, Nfh, rvh, rfh};
+}
 
+// Cheap part of the source, shared by the plain and the surrogate paths: relaxation
+// limiter, moment assembly (Eq. 21), vapour sink (Eqs. 18, 25) and the
+// flux-aware limiters of reading J.  U: conserved stage input of the cell; acc (may be
+// null): its flux-only residual, so that the limiters act on A = U + dt acc.  BI: the
+// bimodal liquid, whose second set (fields 14..17) takes the heterogeneous nucleation
+// r.Jh, grows at r.Gh and alone freezes by immersion.
+template <class T, bool BI = false>
+__device__ __forceinline__ void source_assemble(const Prim<T>& w, const T* U, const T* acc, T dt, const SrcCase& sc,
+                                            const Freezing<T>& fz, Rates<T> r, T* Q, double* aux) {
+  const T rho = w.rho;
+  // growth over the stage: the exponential solution of the linearised exchange
+  const T xsum = BI ? dt * (r.xl + r.xh + r.xs) : dt * (r.xl + r.xs);
+  if (xsum > T(0)) {
+    const T theta = m_div(-m_expm1(-xsum), xsum);
+    r.Gl *= theta;
+    r.Gs *= theta;
+    if (BI) r.Gh *= theta;
+  }
+  if (aux) { aux[7] = double(r.Gl) * 1e-6; aux[8] = double(r.Gs) * 1e-6; }
+
+  const T Nf = fz.Nf, rv = fz.rv, rf = fz.rf, Nfh = fz.Nfh, rvh = fz.rvh, rfh = fz.rfh;
   // moment sources (per kg, scaled units), Eq. (21)
   const T jr = m_div(r.Jeff, rho);
   T dml[4], dms[4], dmh[4];
@@ -571,6 +588,15 @@ __device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const 
     Q[9 + q] = rho * dms[q];
     if (BI) Q[14 + q] = rho * dmh[q];
   }
+}
+
+// the freezing and the assembly in one
+template <class T, bool BI = false>
+__device__ __forceinline__ void source_tail(const Prim<T>& w, const T* U, const T* acc, T dt, const SrcCase& sc,
+                                            bool pres_l, bool pres_s, double lnSl, double lnSi, const Rates<T>& r, T* Q,
+                                            double* aux, bool pres_h = false) {
+  const Freezing<T> fz = freezing_rates<T, BI>(w, dt, sc, pres_l, pres_h, lnSl, lnSi, aux);
+  source_assemble<T, BI>(w, U, acc, dt, sc, fz, r, Q, aux);
 }
 
 // Saturation state of a cell (Eq. 1, FP64): ln S over liquid and ice, ln p_v, populations.
@@ -664,8 +690,8 @@ __device__ __forceinline__ T kantrowitz_phi(const Prim<T>& w, const Gas<T>& g, d
                (T(k::ALPHA_Y - 0.5) - m_div(T(0.5) * (g.gam_g + T(1)), T(2) * g.gam_g) * g.cp_g * Tsat_l * ih);
   const T Knc = m_div(g.lbar, T(2) * rcT);
   const T alpha_c = m_div(g.lam, rcT * (T(1) + T(3.78) * (T(1) - nu) * Knc * T(1.0 / k::PR)));
-  return m_div(T(k::QC) * T(rhov), alpha_c) * m_sqrt(T(k::RV) * Tg * T(1.0 / (2.0 * k::PI))) *
-         (m_div(g.hfg * g.hfg, T(k::RV) * Tg * Tg) - m_div(g.hfg, Tg));
+  return own_mul(m_div(T(k::QC) * T(rhov), alpha_c) * m_sqrt(T(k::RV) * Tg * T(1.0 / (2.0 * k::PI))),
+                 m_div(g.hfg * g.hfg, T(k::RV) * Tg * Tg) - m_div(g.hfg, Tg));
 }
 
 // Classical nucleation, Eqs. (3), (4), (9), (10), with the soot gate of J_het (reading F):
@@ -675,13 +701,17 @@ __device__ __forceinline__ T kantrowitz_phi(const Prim<T>& w, const Gas<T>& g, d
 struct Cnt {
   double rc, rhov, Jhom, Jhet, Jsum;
 };
+// critical radius: surface tension sigd, reciprocal temperature iT
+__device__ __forceinline__ double kelvin_radius(double sigd, double iT, double lnSl) {
+  return sigd * iT * m_div(2.0 / (k::RHOL * k::RV), lnSl);
+}
 template <class T>
 __device__ __forceinline__ Cnt cnt_rates(const Prim<T>& w, double lnSl, const SrcCase& sc, double* lnJ2) {
   const T Tg = w.Tg, rho = w.rho;
   Cnt c;
   const T sig = prop_sigma<T>(sc, Tg);
   const double sigd = to_d(sig), iT = rcp_t(to_d(Tg));
-  c.rc = sigd * iT * m_div(2.0 / (k::RHOL * k::RV), lnSl);
+  c.rc = kelvin_radius(sigd, iT, lnSl);
   const double dGkT = (k::FOUR_PI_3 / k::KB) * iT * sigd * c.rc * c.rc;
   c.rhov = to_d(rho) * to_d(w.Yv);
   // ln A = ln q_c + 1/2 ln(2 sigma N_A^3 / (pi M^3)) + 2 ln rho_v - ln rho_l
@@ -704,6 +734,24 @@ __device__ __forceinline__ Cnt cnt_rates(const Prim<T>& w, double lnSl, const Sr
   return c;
 }
 
+// Growth at r20 of a liquid set m and of the ice, Eqs. (16), (21): G in um/s and the relaxation rate
+// of reading J; Tsat, lnS: of the phase.
+template <class T>
+__device__ __forceinline__ void liquid_growth(const Prim<T>& w, const T* m, const Gas<T>& gs, T Tsat, double lnS, const SrcCase& sc,
+                                              T& G, T& x) {
+  const T r20 = m_sqrt(m_div(m[2], m[0])) * T(1e-6);
+  const Growth<T> g = young_growth<T>(r20, w.Tg, Tsat, T(lnS), prop_sigma<T>(sc, w.Tg), T(k::RHOL), gs.hfg, gs.lam, gs.lbar, gs.gam_g, gs.cp_g);
+  G = g.cond * g.D * T(1e6);
+  x = own_mul(T(4.0 * k::PI * k::RHOL * 1e-12) * m[2] * g.cond, relax_slope(Tsat, w.Tg, gs.hfg, w.Yv, w.cv));
+}
+template <class T>
+__device__ __forceinline__ void ice_growth(const Prim<T>& w, const Gas<T>& gs, T Tsat, double lnS, T& G, T& x) {
+  const T r20 = m_sqrt(m_div(w.ms[2], w.ms[0])) * T(1e-6);
+  const Growth<T> g = young_growth<T>(r20, w.Tg, Tsat, T(lnS), T(k::SIGMA_SV), T(k::RHOS), gs.hsg, gs.lam, gs.lbar, gs.gam_g, gs.cp_g);
+  G = g.cond * g.D * T(1e6);
+  x = own_mul(T(4.0 * k::PI * k::RHOS * 1e-12) * w.ms[2] * g.cond, relax_slope(Tsat, w.Tg, gs.hsg, w.Yv, w.cv));
+}
+
 // Plain rates, Sec. 2.2.  ext (optional, the surrogate's training targets): 0 ln Jeff,
 // 1 ln r_crit/um, 2 G_l raw (um/s), 3 G_s raw, 4 1/tau_l, 5 1/tau_s, 6 ln J_hom,
 // 7 ln J_het,eff, 8 ln(1+phi), 9 T_sat,l - T.
@@ -713,7 +761,6 @@ __device__ __forceinline__ Rates<T> plain_rates(const Prim<T>& w, const Sat<T>& 
   const T Tg = w.Tg;
   Rates<T> r = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
   const Gas<T> gs = gas_props<T>(w);
-  const T cp_g = gs.cp_g, gam_g = gs.gam_g, lam = gs.lam, lbar = gs.lbar, hfg = gs.hfg, hsg = gs.hsg;
   const T lnpv_t = T(st.lnpv);
   const double lnSl = st.lnSl, lnSi = st.lnSi;
 
@@ -744,26 +791,10 @@ __device__ __forceinline__ Rates<T> plain_rates(const Prim<T>& w, const Sat<T>& 
     }
   }
 
-  // growth at r20, Eqs. (16), (21) -- G in um/s, relaxation rates of reading J
-  if (st.pres_l) {
-    const T r20 = m_sqrt(m_div(w.ml[2], w.ml[0])) * T(1e-6);
-    const Growth<T> g = young_growth<T>(r20, Tg, Tsat_l, T(lnSl), prop_sigma<T>(sc, Tg), T(k::RHOL), hfg, lam, lbar, gam_g, cp_g);
-    r.Gl = g.cond * g.D * T(1e6);
-    r.xl = T(4.0 * k::PI * k::RHOL * 1e-12) * w.ml[2] * g.cond * relax_slope(Tsat_l, Tg, hfg, w.Yv, w.cv);
-  }
-  if (BI && st.pres_h) {
-    const T r20 = m_sqrt(m_div(w.mh[2], w.mh[0])) * T(1e-6);
-    const Growth<T> g = young_growth<T>(r20, Tg, Tsat_l, T(lnSl), prop_sigma<T>(sc, Tg), T(k::RHOL), hfg, lam, lbar, gam_g, cp_g);
-    r.Gh = g.cond * g.D * T(1e6);
-    r.xh = T(4.0 * k::PI * k::RHOL * 1e-12) * w.mh[2] * g.cond * relax_slope(Tsat_l, Tg, hfg, w.Yv, w.cv);
-  }
-  if (st.pres_s) {
-    const T Tsat_i = prop_tsat<T, true>(sc, lnpv_t);
-    const T r20 = m_sqrt(m_div(w.ms[2], w.ms[0])) * T(1e-6);
-    const Growth<T> g = young_growth<T>(r20, Tg, Tsat_i, T(lnSi), T(k::SIGMA_SV), T(k::RHOS), hsg, lam, lbar, gam_g, cp_g);
-    r.Gs = g.cond * g.D * T(1e6);
-    r.xs = T(4.0 * k::PI * k::RHOS * 1e-12) * w.ms[2] * g.cond * relax_slope(Tsat_i, Tg, hsg, w.Yv, w.cv);
-  }
+  // growth at r20
+  if (st.pres_l) liquid_growth<T>(w, w.ml, gs, Tsat_l, lnSl, sc, r.Gl, r.xl);
+  if (BI && st.pres_h) liquid_growth<T>(w, w.mh, gs, Tsat_l, lnSl, sc, r.Gh, r.xh);
+  if (st.pres_s) ice_growth<T>(w, gs, prop_tsat<T, true>(sc, lnpv_t), lnSi, r.Gs, r.xs);
   if (ext) {
     ext[2] = double(r.Gl);
     ext[3] = double(r.Gs);
@@ -799,6 +830,78 @@ __device__ __forceinline__ void mlp_features(const Prim<T>& w, const Sat<T>& st,
   x[13] = logf(float(rp2 * 1e12) + 1e-30f);
   x[14] = float(st.lnSl);
   x[15] = float(st.lnSi);
+}
+
+// The flux-free parts of one cell's source in four shares (T in FP64, one liquid set), for four warps
+// of a small tile: 0 the freezing, 1 the nucleation rates, 2 the liquid's growth with the
+// Kantrowitz factor, 3 the ice's growth.  The expressions are those of saturation, plain_rates
+// and freezing_rates.  out[q * stride], q = SH_*; flags (share 2 only): SF_* bits.
+enum { SH_NF, SH_RV, SH_RF, SH_J, SH_LNJ0, SH_LNJ1, SH_GL, SH_XL, SH_PHI, SH_RC, SH_GS, SH_XS, NSHARE };
+enum { SF_ACTIVE = 1, SF_NUCLEATES = 2 };
+template <class T>
+__device__ __forceinline__ void source_share(int share, const Prim<T>& w, T dt, const SrcCase& sc, T* out, int stride, int* flags) {
+  bool pl, ps;
+  const bool idle = !populations(w, pl, ps) && clearly_inactive(w);
+  Sat<T> st;
+  st.active = false;
+  if (!idle) st = saturation<T, false>(w, sc);
+  if (!st.active) {
+    if (share == 2) *flags = 0;
+    return;
+  }
+  const bool nuc = st.lnSl > 0.0;
+  if (share == 0) {
+    const Freezing<T> fz = freezing_rates<T, false>(w, dt, sc, st.pres_l, false, st.lnSl, st.lnSi, nullptr);
+    out[SH_NF * stride] = fz.Nf;
+    out[SH_RV * stride] = fz.rv;
+    out[SH_RF * stride] = fz.rf;
+  } else if (share == 1) {
+    if (!nuc) return;
+    double lnJ2[2] = {-INFINITY, -INFINITY};
+    out[SH_J * stride] = T(cnt_rates<T>(w, st.lnSl, sc, lnJ2).Jsum);
+    out[SH_LNJ0 * stride] = T(lnJ2[0]);
+    out[SH_LNJ1 * stride] = T(lnJ2[1]);
+  } else if (share == 2) {
+    *flags = SF_ACTIVE | (nuc ? SF_NUCLEATES : 0);
+    T Gl = T(0), xl = T(0);
+    if (nuc || st.pres_l) {
+      const Gas<T> gs = gas_props<T>(w);
+      const T Tsat = prop_tsat<T, false>(sc, T(st.lnpv));
+      if (nuc) {
+        const double rc = kelvin_radius(to_d(prop_sigma<T>(sc, w.Tg)), rcp_t(to_d(w.Tg)), st.lnSl);
+        out[SH_PHI * stride] = kantrowitz_phi<T>(w, gs, rc, to_d(w.rho) * to_d(w.Yv), Tsat);
+        out[SH_RC * stride] = T(rc * 1e6);
+      }
+      if (st.pres_l) liquid_growth<T>(w, w.ml, gs, Tsat, st.lnSl, sc, Gl, xl);
+    }
+    out[SH_GL * stride] = Gl;
+    out[SH_XL * stride] = xl;
+  } else {
+    T Gs = T(0), xs = T(0);
+    if (st.pres_s) ice_growth<T>(w, gas_props<T>(w), prop_tsat<T, true>(sc, T(st.lnpv)), st.lnSi, Gs, xs);
+    out[SH_GS * stride] = Gs;
+    out[SH_XS * stride] = xs;
+  }
+}
+// the source from its shares (see phase_source); lnJ: ln J_hom and ln J_het,eff
+template <class T>
+__device__ __forceinline__ bool source_from_shares(const Prim<T>& w, const T* U, const T* acc, T dt, const SrcCase& sc,
+                                                   const T* in, int stride, int flags, T* Q, T* lnJ) {
+  if (!(flags & SF_ACTIVE)) return false;
+  Rates<T> r = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+  if (flags & SF_NUCLEATES) {
+    r.Jeff = m_div(in[SH_J * stride], T(1) + in[SH_PHI * stride]);
+    r.rc_um = in[SH_RC * stride];
+    lnJ[0] = in[SH_LNJ0 * stride];
+    lnJ[1] = in[SH_LNJ1 * stride];
+  }
+  r.Gl = in[SH_GL * stride];
+  r.xl = in[SH_XL * stride];
+  r.Gs = in[SH_GS * stride];
+  r.xs = in[SH_XS * stride];
+  const Freezing<T> fz = {in[SH_NF * stride], in[SH_RV * stride], in[SH_RF * stride], T(0), T(0), T(0)};
+  source_assemble<T, false>(w, U, acc, dt, sc, fz, r, Q, nullptr);
+  return true;
 }
 
 // Source of one cell (plain method).  w: primitives of the stage input; the limiters keep

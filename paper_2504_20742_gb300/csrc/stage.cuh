@@ -801,6 +801,39 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
 
   const T dt = s_dt;
 
+  // primitives of the tile's cell (ci, cj), cell n of the grid: SP: the stencil's from shared memory,
+  // T and c_v stored
+  const auto load_prims = [&](int ci, int cj, size_t n, Prim<T>& w) {
+    if constexpr (SP) {
+      w.rho = qs(0, cj + 2, ci + 2);
+      w.u = qs(1, cj + 2, ci + 2);
+      w.v = qs(2, cj + 2, ci + 2);
+      w.p = qs(3, cj + 2, ci + 2);
+      w.Yv = qs(4, cj + 2, ci + 2);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        w.ml[q] = qs(5 + q, cj + 2, ci + 2);
+        w.ms[q] = qs(9 + q, cj + 2, ci + 2);
+      }
+      w.ns = qs(13, cj + 2, ci + 2);
+      w.Yl = rn_mul(T(k::YL3), w.ml[3]);   // as the conversion forms them
+      w.Ys = rn_mul(T(k::YS3), w.ms[3]);
+      const T* src = reinterpret_cast<const T*>(dc.prims) + (STAGE == 1 ? 0 : (size_t)NPLANE * N);
+      w.Tg = src[NFX * N + n];
+      w.cv = src[(NFX + 1) * N + n];
+      w.Rg = w.c2 = T(0);   // not used by the cell update
+    } else {
+      T u[NFX];
+#pragma unroll
+      for (int f = 0; f < NFX; ++f) u[f] = Uin[f * N + n];
+      cons_to_prim<T, BI>(u, w);
+    }
+  };
+  // small FP64 tiles: the source's shares (source_share)
+  constexpr bool SHARES = TL::SEP && IS64 && !SURR && !BI;
+  __shared__ T s_share[SHARES ? NSHARE : 1][32];
+  __shared__ int s_flags[32];
+
   // phase B1: limited x slopes, once per cell, written as the states of its two faces
   // (tile-local cell c in [-1, TX]; face f lies between cells f-1 and f): cell p, pairs k_lo .. k_hi - 1
   constexpr int NSX = (TX + 2) * TY, NSR = TX * (TY + 2);
@@ -918,6 +951,17 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
           r_flux(p - XW, t);
       }
     });
+    // The parts of the source that take nothing from the fluxes, a share per warp after (or beside)
+    // its fluxes: @@C@@
+    if constexpr (SHARES) {
+      static_assert(NT == 128 && NCELL <= 32, "four shares, a lane per cell");
+      const int c = tid & 31, ci = c % TX, cj = c / TX, i = i0 + ci, j = j0 + cj;
+      if (dc.sc.phase_change && !dc.sc.equilibrium && c < NCELL && i < nx && j < nr) {
+        Prim<T> w;
+        load_prims(ci, cj, (size_t)j * nx + i, w);
+        source_share<T>(tid >> 5, w, dt, dc.sc, &s_share[0][c], 32, &s_flags[c]);
+      }
+    }
   } else {
     with_dry([&](auto t) {
       if constexpr (TL::ITEMS) {
@@ -1043,27 +1087,8 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     const size_t n = (size_t)j * nx + i;
 #pragma unroll
     for (int f = 0; f < NFX; ++f) u14[f] = Uin[f * N + n];
-    if (SP) {   // the cell's primitives: the stencil's from shared memory, T and c_v stored
-      w.rho = qs(0, cj + 2, ci + 2);
-      w.u = qs(1, cj + 2, ci + 2);
-      w.v = qs(2, cj + 2, ci + 2);
-      w.p = qs(3, cj + 2, ci + 2);
-      w.Yv = qs(4, cj + 2, ci + 2);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        w.ml[q] = qs(5 + q, cj + 2, ci + 2);
-        w.ms[q] = qs(9 + q, cj + 2, ci + 2);
-      }
-      w.ns = qs(13, cj + 2, ci + 2);
-      w.Yl = rn_mul(T(k::YL3), w.ml[3]);   // as the conversion forms them
-      w.Ys = rn_mul(T(k::YS3), w.ms[3]);
-      const T* src = reinterpret_cast<const T*>(dc.prims) + (STAGE == 1 ? 0 : (size_t)NPLANE * N);
-      w.Tg = src[NFX * N + n];
-      w.cv = src[(NFX + 1) * N + n];
-      w.Rg = w.c2 = T(0);   // not used by the cell update
-    } else {
-      cons_to_prim<T, BI>(u14, w);
-    }
+    if constexpr (SP) load_prims(ci, cj, n, w);
+    else cons_to_prim<T, BI>(u14, w);
     if (dc.geom == 1) {
       T ijh, cs, cn;
       bool wall;
@@ -1125,7 +1150,18 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     T Q[NFX];
     double lnJ2[2];
     if (!SURR) {
-      const bool act = phase_source<T, BI>(w, u14, acc, dt, dc.sc, Q, lnJ2, nullptr);
+      bool act = false;
+      if constexpr (SHARES) {
+        if (dc.sc.phase_change && dc.sc.equilibrium) {
+          act = equilibrium_source<T>(u14, acc, dt, dc.sc, Q, nullptr);
+          lnJ2[0] = lnJ2[1] = -INFINITY;
+        } else if (dc.sc.phase_change) {
+          lnJ2[0] = lnJ2[1] = -INFINITY;
+          act = source_from_shares<T>(w, u14, acc, dt, dc.sc, &s_share[0][tid], 32, s_flags[tid], Q, lnJ2);
+        }
+      } else {
+        act = phase_source<T, BI>(w, u14, acc, dt, dc.sc, Q, lnJ2, nullptr);
+      }
       nactive = act ? 1 : 0;
       // inactive cells keep -inf without a conversion, and their source is +0: adding it
       // could only turn a -0 into +0, which the update cannot tell apart
