@@ -366,8 +366,13 @@ __device__ inline bool last_block_reduce(const DevCase& dc, double* out, double*
 // row's records into a row record, and the last row to complete reduces the row records.
 // Both orders are fixed, so the totals are deterministic; no CTA waits for another, and
 // the serial part on the critical path is one row of records instead of all of them.
+// One level for a single row of tiles and for up to ONE_LEVEL tiles in all, where a second ticket, its
+// fences and the reload of the row records take longer than the records themselves (the nozzle's 50
+// tiles: 11,800 cycles, two levels 16,100).
+constexpr int ONE_LEVEL = 64;
 // `by`: this tile's row; scratch as reduce_records.  Returns true in the CTA that completed the case.
 __device__ inline bool tile_reduce(const DevCase& dc, int by, double* out, double* scratch) {
+  if (dc.nblocks <= ONE_LEVEL || dc.tiles_y == 1) return last_block_reduce(dc, out, scratch);
   __shared__ unsigned int ticket;
   if (threadIdx.x < NPART) __threadfence();   // the record's writers publish it
   __syncthreads();
@@ -800,7 +805,33 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   const bool dry = DRY_OK ? __syncthreads_and(zb == 0u) != 0 : (__syncthreads(), false);
 
   const T dt = s_dt;
+  // quasi-1D: areas of the faces of column i, their weights in the divergence, the cell volume
+  const auto nozzle_geometry = [&](int i, T& area_w, T& area_e, T& cw, T& ce, T& vol) {
+    const T xw = T(i) * g.dx, xe = T(i + 1) * g.dx, xc = (T(i) + T(0.5)) * g.dx;
+    const T sw = xw * g.ixt - T(1), se = xe * g.ixt - T(1), sc = xc * g.ixt - T(1);
+    area_w = T(1) + g.area_a * sw * sw;
+    area_e = T(1) + g.area_a * se * se;
+    const T Ac = T(1) + g.area_a * sc * sc;
+    const T iv = trcp(Ac * g.dx);
+    cw = area_w * iv;
+    ce = area_e * iv;
+    vol = Ac * g.dx;
+  };
 
+  constexpr bool SHARES = TL::SEP && IS64 && !SURR && !BI;
+  T u_early[SHARES ? NFX : 1], un_early[SHARES && STAGE == 2 ? NFX : 1];
+  if constexpr (SHARES) {
+    const int i = i0 + tid % TX, j = j0 + tid / TX;
+    if (tid < NCELL && i < nx && j < nr) {
+      const size_t n = (size_t)j * nx + i;
+#pragma unroll
+      for (int f = 0; f < NFX; ++f) u_early[f] = Uin[f * N + n];
+      if constexpr (STAGE == 2) {
+#pragma unroll
+        for (int f = 0; f < NFX; ++f) un_early[f] = Un[f * N + n];
+      }
+    }
+  }
   // primitives of the tile's cell (ci, cj), cell n of the grid: SP: the stencil's from shared memory,
   // T and c_v stored
   const auto load_prims = [&](int ci, int cj, size_t n, Prim<T>& w) {
@@ -829,10 +860,13 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
       cons_to_prim<T, BI>(u, w);
     }
   };
-  // small FP64 tiles: the source's shares (source_share)
-  constexpr bool SHARES = TL::SEP && IS64 && !SURR && !BI;
+  // small FP64 tiles: the source's shares (source_share), and the states of the cell update asked for
+  // before the fluxes (with the nozzle's geometry in a share and one-level totals: 3725 -> 3490 us for
+  // 50 steps of the 400-cell nozzle)
   __shared__ T s_share[SHARES ? NSHARE : 1][32];
   __shared__ int s_flags[32];
+  // quasi-1D geometry of the tile's columns: west and east areas, weights, volume, dA/V
+  __shared__ T s_col[SHARES ? 6 : 1][TX];
 
   // phase B1: limited x slopes, once per cell, written as the states of its two faces
   // (tile-local cell c in [-1, TX]; face f lies between cells f-1 and f): cell p, pairs k_lo .. k_hi - 1
@@ -952,10 +986,23 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
       }
     });
     // The parts of the source that take nothing from the fluxes, a share per warp after (or beside)
-    // its fluxes: @@C@@
+    // its fluxes.  FP64 instructions bound a stage here, one after another in the cell's warp (64 cycles
+    // each): with saturation, nucleation, growth and freezing in that warp after the fluxes, 50 steps
+    // of the 400-cell nozzle took 4185 us, with the shares 3697 us; 20 steps of a freezing plume of
+    // 77 x 29 cells 2104 and 1745 us.  The nozzle's geometry goes to the warp without liquid or faces.
     if constexpr (SHARES) {
       static_assert(NT == 128 && NCELL <= 32, "four shares, a lane per cell");
       const int c = tid & 31, ci = c % TX, cj = c / TX, i = i0 + ci, j = j0 + cj;
+      if (dc.geom == 0 && tid >= 96 && c < TX) {
+        T aw, ae, cw, ce, vol;
+        nozzle_geometry(i, aw, ae, cw, ce, vol);
+        s_col[0][c] = aw;
+        s_col[1][c] = ae;
+        s_col[2][c] = cw;
+        s_col[3][c] = ce;
+        s_col[4][c] = vol;
+        s_col[5][c] = tdiv(ae - aw, vol);
+      }
       if (dc.sc.phase_change && !dc.sc.equilibrium && c < NCELL && i < nx && j < nr) {
         Prim<T> w;
         load_prims(ci, cj, (size_t)j * nx + i, w);
@@ -997,15 +1044,15 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
     const int w = cj * (TX + 1) + ci, e = w + 1;
     T cw, ce;
     if (dc.geom == 0) {
-      const T xw = T(i) * g.dx, xe = T(i + 1) * g.dx, xc = (T(i) + T(0.5)) * g.dx;
-      const T sw = xw * g.ixt - T(1), se = xe * g.ixt - T(1), sc = xc * g.ixt - T(1);
-      area_w = T(1) + g.area_a * sw * sw;
-      area_e = T(1) + g.area_a * se * se;
-      const T Ac = T(1) + g.area_a * sc * sc;
-      const T iv = trcp(Ac * g.dx);
-      cw = area_w * iv;
-      ce = area_e * iv;
-      vol = Ac * g.dx;
+      if constexpr (SHARES) {
+        area_w = s_col[0][ci];
+        area_e = s_col[1][ci];
+        cw = s_col[2][ci];
+        ce = s_col[3][ci];
+        vol = s_col[4][ci];
+      } else {
+        nozzle_geometry(i, area_w, area_e, cw, ce, vol);
+      }
     } else {
       cw = ce = g.idx;
       if constexpr (IS64) {
@@ -1086,7 +1133,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   if (cell) {
     const size_t n = (size_t)j * nx + i;
 #pragma unroll
-    for (int f = 0; f < NFX; ++f) u14[f] = Uin[f * N + n];
+    for (int f = 0; f < NFX; ++f) u14[f] = SHARES ? u_early[SHARES ? f : 0] : Uin[f * N + n];
     if constexpr (SP) load_prims(ci, cj, n, w);
     else cons_to_prim<T, BI>(u14, w);
     if (dc.geom == 1) {
@@ -1144,7 +1191,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
         be -= An * gb(3, e);
       }
     } else {
-      acc[1] += w.p * tdiv(area_e - area_w, vol);
+      acc[1] += w.p * (SHARES ? s_col[SHARES ? 5 : 0][ci] : tdiv(area_e - area_w, vol));
     }
     // phase-change source limited on the flux-updated state
     T Q[NFX];
@@ -1183,6 +1230,10 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
   if (cell) {
     const size_t n = (size_t)j * nx + i;
     // RK combine
+    const auto un_of = [&](int f, size_t n) -> T {
+      if constexpr (SHARES && STAGE == 2) return un_early[f];
+      else return Un[f * N + n];
+    };
     T out[NFX];
     const V dt2 = p_make(dt, dt);
     // FP64: moment fields that are +0 in the input states with a zero rate stay +0 (exactly
@@ -1202,7 +1253,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
           T unm[NFX];
 #pragma unroll
           for (int f = 0; f < NFX; ++f)
-            if (is_moment(f)) unm[f] = Un[f * N + n];
+            if (is_moment(f)) unm[f] = un_of(f, n);
           mz = bits0(unm);
         }
       }
@@ -1233,7 +1284,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
 #pragma unroll
       for (int f = 0; f < NFX; ++f) {
         if (is_moment(f)) continue;
-        const T un = Un[f * N + n];
+        const T un = un_of(f, n);
         out[f] = fma(T(0.5), un, half_of(fma(dt, acc[f], u14[f])));
         if (f < NF) rmax[f] = m_fabs(out[f] - un);   // divided by dt once per CTA
       }
@@ -1248,7 +1299,7 @@ __device__ __forceinline__ void stage_tile(const DevCase& dc, int bx, int by, in
 #pragma unroll
         for (int f = 0; f < NFX; ++f) {
           if (!is_moment(f)) continue;
-          const T un = Un[f * N + n];
+          const T un = un_of(f, n);
           out[f] = fma(T(0.5), un, half_of(fma(dt, acc[f], u14[f])));
           const T rf = m_fabs(out[f] - un);
           if (f < NF) {
