@@ -97,19 +97,19 @@ def _workload(name):
 
 
 # Per-cell figures of the fused stage kernel, from one ncu capture each (see profiles/):
-# FP64 arithmetic per cell-stage executed on the plume (mean of the two stages, 527.9 and
-# 602.2 flops on the 16 x 16 two-CTA tile; the kernels skip the exact zeros of the particle
+# FP64 arithmetic per cell-stage executed on the plume (mean of the two stages, 451.5 and
+# 511.5 flops on the 16 x 16 two-CTA tile; the kernels skip the exact zeros of the particle
 # moments in air without liquid or ice), and DRAM bytes per cell per launch (mean of the two stages) by tile shape,
 # reported only for a shape counted on the current kernel.
-FP64_FLOPS_PER_CELL_STAGE = 565.1
-FP64_TRAFFIC_PER_CELL_LAUNCH = {7: 452.0}    # 16 x 16, two CTAs per SM
+FP64_FLOPS_PER_CELL_STAGE = 481.5
+FP64_TRAFFIC_PER_CELL_LAUNCH = {6: 399.2, 7: 455.6, 8: 397.9}    # 16 x 12, 16 x 16, 16 x 15, two CTAs per SM
 FP32_TRAFFIC_PER_CELL_LAUNCH = {9: 140.4}    # the column sweep (28 x 64 strips), four CTAs per SM
 SWEEP_SHAPE = 9   # tile shape index of the column-sweep FP32 kernel (k_sweep)
-# the viscous FP64 kernel (same capture recipe, plume with nu_t = 0.5 m^2/s, 16 x 14 tile:
-# 1135.9 and 1377.4 flops)
-FP64_VISC_FLOPS_PER_CELL_STAGE = 1256.7
-# the bimodal FP64 kernel (18 fields; same recipe, dormant plume: 576.3 and 688.6 flops)
-FP64_BI_FLOPS_PER_CELL_STAGE = 632.5
+# the viscous FP64 kernel (same capture recipe, plume with nu_t = 0.5 m^2/s, 16 x 16 two-CTA tile:
+# 865.2 and 1009.1 flops)
+FP64_VISC_FLOPS_PER_CELL_STAGE = 937.2
+# the bimodal FP64 kernel (18 fields; same recipe, dormant plume: 488.5 and 578.8 flops)
+FP64_BI_FLOPS_PER_CELL_STAGE = 533.7
 
 
 def measure_dgemm_tflops(dev) -> float:
@@ -300,7 +300,7 @@ def run_cuda(args):
                 "kernel": "ct::k_stage<double>",
                 "peak_source": "measured: cuBLAS DGEMM 4096^3 on this GPU (FP64 has no entry in MEASURED_PEAKS.json)",
                 "note": f"{per_cell} FP64 flops per cell-stage executed (a DFMA counts 2, a DADD or DMUL 1; "
-                        "the FP64 pipe was 76-78 % busy on the plume in the ncu capture, profiles/); "
+                        "the FP64 pipe was 75-76 % busy on the plume in the ncu capture, profiles/); "
                         "the peak is cuBLAS DGEMM timed in this run; traffic (DRAM bytes of the ncu capture) "
                         "exceeds the 280 algorithmic bytes per cell-launch because the kernel reads and "
                         "writes the stored primitive planes on purpose (DRAM 2-3 % busy); "
