@@ -393,9 +393,9 @@ static std::tuple<int, int, int, int> shape_key(const ct_case* c, int precision)
   return std::make_tuple(c->geom, c->nx, case_nr(c), variant_of(c, precision));
 }
 // Without a registered shape: 32 x 8 tiles, or for plain FP64 on grids that leave SMs without one
-// the small tiles: 8 x 2 up to 400 of them (a step of the freezing plume 77 x 29: 251 us with 32 x 8
-// tiles, 115 with 8 x 4, 111 with 8 x 2; 150 x 40: 265, 126, 118), 8 x 4 beyond (256 x 64 cells, 1,024
-// tiles of 8 x 2: 194 against 260).  FP32 keeps 32 x 8, so that its totals, summed in FP32 within a
+// the small tiles: 8 x 2 up to 400 of them (a step of the freezing plume 77 x 29: 232 us with 32 x 8
+// tiles, 96 with 8 x 4, 87 with 8 x 2; 150 x 40: 247, 103, 98), 8 x 4 beyond (a condensing plume of
+// 256 x 64 cells, 1,024 tiles of 8 x 2: 188 against 241).  FP32 keeps 32 x 8, so that its totals, summed in FP32 within a
 // warp, are those of a batch's cases; the autotuner may choose the small tiles there.
 static int default_shape(const ct_case* c, int precision) {
   if (variant_of(c, precision) != 0 || cells_of(c) > SMALL_GRID) return 0;

@@ -1531,8 +1531,9 @@ struct StageSet {
   bool small_grid;                  // for grids of at most SMALL_GRID cells only
 };
 // Largest grid the small tiles serve, in cells.  A step of the freezing plume in FP64 on GB300, 32 x 8
-// tiles / 8 x 4 tiles: 300 x 80 cells 268 / 181 us, a condensing plume 256 x 64 277 / 194 us; on
-// 400 x 100 cells, which give every SM a 32 x 8 tile, 263 / 264 and 280 / 376 us.
+// tiles / 8 x 4 tiles: a condensing plume 256 x 64 256 / 188 us (300 x 80 cells 268 / 181 before
+// the source's shares); on 400 x 100 cells, which give every SM a 32 x 8 tile, 263 / 264 and 280 / 376
+// before them, 243 and 258 with 32 x 8 tiles now.
 constexpr size_t SMALL_GRID = 20480;
 constexpr size_t SMEM_LIMIT = 227 * 1024 - 4096;   // opt-in limit minus the static shared memory
 

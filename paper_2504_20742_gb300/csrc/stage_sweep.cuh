@@ -572,7 +572,8 @@ __global__ void __launch_bounds__(ST::NT, ST::MINB)
 // on the device only.  Its three warpgroups never wait for one another, so the FP64 islands and
 // FP32 work of one run beside the network layers of the others.  (Two CTAs of 256 threads per SM
 // that streamed the weights layer by layer and compacted the surrogate cells of both their halves
-// into one tile took 223 us for the 155,000 kept cells of a 1024 x 256 plume's stage.)
+// into one tile took 223 us for the 155,000 kept cells of a 1024 x 256 plume's stage; this form
+// 104 us, with the FP64 functions of logexp.cuh.)
 // The queue of one case (all threads of every CTA of the launch; pub: the CTA that publishes the
 // stage when nothing is queued).  phase: the group's tensor-core barrier phase.
 template <int STAGE>
