@@ -50,6 +50,23 @@ def test_same_bits_as_the_default_tile(P, prec, nx, nr):
             assert abs(d[q] - d0[q]) <= (1e-12 if prec == 0 else 1e-5) * abs(d0[q])
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("opt", [dict(tables=1), dict(equilibrium=1), dict(phase_change=0), dict(freezing=0), dict(viscous=1, nu_t=0.05),
+                                 dict(n_soot=0.0)])
+@pytest.mark.parametrize("nx,nr", [(33, 31), (9, 5), (64, 24)])
+def test_same_bits_with_the_model_options(P, nx, nr, opt):
+    """The source's shares of the small FP64 tiles and the totals in one level (up to 64 tiles) or two."""
+    c, uf = cases.mixing_layer_case(nx=nx, nr=nr)
+    c = dict(c, **opt)
+    ref, d0 = _run(P, c, uf, 0, 0, 5)
+    for k in _shapes(P, 0):
+        U, d = _run(P, c, uf, 0, k, 5)
+        assert torch.equal(U.view(torch.int64), ref.view(torch.int64)), k
+        assert d[0] == d0[0] and d[7] == d0[7] and np.array_equal(d[9:25], d0[9:25])
+        for q in (1, 2, 3):
+            assert abs(d[q] - d0[q]) <= 1e-12 * abs(d0[q])
+
+
 def test_small_tiles_are_refused_on_large_grids(P):
     c, _ = cases.plume_case(nx=512, nr=128)
     small = [k for k in range(P.ct_tile_shape_count()) if P.ct_tile_shape(k) in ((8, 4), (8, 2))]
