@@ -154,15 +154,16 @@ __device__ __forceinline__ double ln_psat_of(double T, double lnT, double iT) {
   return ICE ? fma(-0.49382577, lnT, fma(-6024.5282, iT, fma(T, fma(T, -1.3198825e-5, 1.0613868e-2), 24.7219 + k::LN100)))
              : fma(2.433502, lnT, fma(-6096.9385, iT, fma(T, fma(T, 1.673952e-5, -2.711193e-2), 16.635794 + k::LN100)));
 }
-// FP64, the same root: four Newton steps in FP32 (to about 1e-5 K, FP32's resolution of ln p),
-// then two in FP64 with the FP32 slope, whose relative error of 1e-7 leaves the first step at
-// 1e-12 K and the second below rounding.  `lnp` evaluates the curve in FP64.  Six FP64 steps took
-// about 370 FP64-pipe instructions, these take 30 (GB300, one such instruction per 64 issue slots).
-template <bool ICE, class F>
-__device__ __forceinline__ double t_sat_newton(double lnpv, const F& lnp) {
+// FP64, the same root: four Newton steps in FP32 (t_sat_fp32: to about 1e-5 K, FP32's resolution of
+// ln p), then two in FP64 with the FP32 slope, whose relative error of 1e-7 leaves the first step at
+// 1e-12 K and the second below rounding (t_sat_refine; `lnp` evaluates the curve in FP64).  Six FP64
+// steps took about 370 FP64-pipe instructions, these take 30 (GB300, one such instruction per 64 issue
+// slots).
+template <bool ICE>
+__device__ __forceinline__ float t_sat_fp32(double lnpv, float& slope) {
   const float lp = d2f_bits(lnpv);
   float Tf = t_sat_start<float, ICE>(lp);
-  float slope = 1.0f;
+  slope = 1.0f;
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
     const float iT = __fdividef(1.0f, Tf), lnT = __logf(Tf);
@@ -173,6 +174,10 @@ __device__ __forceinline__ double t_sat_newton(double lnpv, const F& lnp) {
     slope = __fdividef(1.0f, slope);
     if (it < 3) Tf = fmaf(lp - f, slope, Tf);
   }
+  return Tf;
+}
+template <class F>
+__device__ __forceinline__ double t_sat_refine(double lnpv, float Tf, float slope, const F& lnp) {
   const double sl = f2d_bits(slope);
   double T = f2d_bits(Tf);
 #pragma unroll
@@ -396,20 +401,34 @@ template <class R>
 __device__ __forceinline__ R prop_sigma(const SrcCase& sc, R T) {
   return sc.tables ? tab_prop(tab_of(sc, R(0)), 2, T, false) : sigma_liq(T);
 }
-// T_sat of reading D with the closed or the tabulated curve (same root in either precision)
+// Six Newton steps on the tabulated curve, with its own slope.
+template <class R, bool ICE>
+__device__ __forceinline__ R t_sat_table(const R* tab, R lnpv) {
+  R T = t_sat_start<R, ICE>(lnpv);
+#pragma unroll
+  for (int it = 0; it < 6; ++it)
+    T -= (tab_prop(tab, ICE ? 1 : 0, T, false) - lnpv) / tab_prop(tab, ICE ? 1 : 0, T, true);
+  return T;
+}
+static __device__ __noinline__ double t_sat_beyond(const double* tab, double lnpv, bool ice) {
+  return ice ? t_sat_table<double, true>(tab, lnpv) : t_sat_table<double, false>(tab, lnpv);
+}
+// T_sat of reading D with the closed or the tabulated curve.  FP64 and tabulated: between the first and
+// the last node (150 and 640 K) the table follows the closed curve to 2e-7 in ln p, so the FP32 root
+// and slope of the closed one serve; outside, where the end node's parabola is another curve (its root
+// up to 30 K from the closed one's at p_v = 1e-30 Pa), the steps are the table's own.
 template <class R, bool ICE>
 __device__ __forceinline__ R prop_tsat(const SrcCase& sc, R lnpv) {
   if constexpr (std::is_same<R, double>::value) {
-    if (sc.tables) return t_sat_newton<ICE>(lnpv, [&](double T) { return tab_prop(sc.tab, ICE ? 1 : 0, T, false); });
-    return t_sat_newton<ICE>(lnpv, [](double T) { return ln_psat_of<ICE>(T, log_t(T), rcp_t(T)); });
+    float slope;
+    const float Tf = t_sat_fp32<ICE>(lnpv, slope);
+    if (sc.tables) {
+      if (!(Tf >= 150.0f && Tf <= 640.0f)) return t_sat_beyond(sc.tab, lnpv, ICE);
+      return t_sat_refine(lnpv, Tf, slope, [&](double T) { return tab_prop(sc.tab, ICE ? 1 : 0, T, false); });
+    }
+    return t_sat_refine(lnpv, Tf, slope, [](double T) { return ln_psat_of<ICE>(T, log_t(T), rcp_t(T)); });
   } else {
-    if (!sc.tables) return t_sat<R, ICE>(lnpv);
-    R T = t_sat_start<R, ICE>(lnpv);
-    const R* tab = tab_of(sc, R(0));
-#pragma unroll
-    for (int it = 0; it < 6; ++it)
-      T -= (tab_prop(tab, ICE ? 1 : 0, T, false) - lnpv) / tab_prop(tab, ICE ? 1 : 0, T, true);
-    return T;
+    return sc.tables ? t_sat_table<R, ICE>(tab_of(sc, R(0)), lnpv) : t_sat<R, ICE>(lnpv);
   }
 }
 
