@@ -357,7 +357,8 @@ ct_status ct_step_static(const ct_case *c, int precision, const double *ufac_row
  * The fused stage kernel is built for several tile shapes (cells per CTA); the state a step
  * produces does not depend on the shape, only the speed does.  Steps of a case use the
  * shape registered for its (geometry, nx, nr, precision), else shape 0 (32 x 8), or in plain
- * CT_FP64 on small grids (up to 20,480 cells) one of the small tiles (8 x 4, 8 x 2). */
+ * CT_FP64 one of the small tiles (8 x 4, 8 x 2) on small grids that step faster by them (up to
+ * 20,480 cells; nozzles up to 912). */
 
 /* Number of tile shapes the library is built with. */
 int ct_tile_shape_count(void);

@@ -392,13 +392,29 @@ static std::map<std::tuple<int, int, int, int>, int> g_shape;
 static std::tuple<int, int, int, int> shape_key(const ct_case* c, int precision) {
   return std::make_tuple(c->geom, c->nx, case_nr(c), variant_of(c, precision));
 }
-// Without a registered shape: 32 x 8 tiles, or for plain FP64 on grids that leave SMs without one
-// the small tiles: 8 x 2 up to 400 of them (a step of the freezing plume 77 x 29: 232 us with 32 x 8
-// tiles, 96 with 8 x 4, 87 with 8 x 2; 150 x 40: 247, 103, 98), 8 x 4 beyond (a condensing plume of
-// 256 x 64 cells, 1,024 tiles of 8 x 2: 188 against 241).  FP32 keeps 32 x 8, so that its totals, summed in FP32 within a
-// warp, are those of a batch's cases; the autotuner may choose the small tiles there.
+// Without a registered shape: 32 x 8 tiles, or for plain FP64 the small tiles where they are faster.
+// What a stage of small tiles takes grows with its tiles (two per SM at a time) and with the records
+// that its last CTAs add up one after another, a row of tiles and then the rows: some 0.17 us a step for
+// each.  A stage of up to 152 tiles of 32 x 8 takes the same time for any number.  So the line is at
+// load = tiles + tiles in a row + rows of tiles (us a step, GB300; plumes: 8 x 4 / 32 x 8 tiles):
+//   load        condensing  dormant         load         condensing  dormant
+//    675 200x100  207 / 258  132 / 117       752 2000x8    268 / 217  150 / 107
+//    721 290x70   215 / 258  134 / 117       801 3200x4    254 / 154  153 /  83
+//    728 64x320   218 / 259  143 / 117      1027 2048x10   274 / 228  169 / 112
+// A young plume without condensate (which the host cannot tell) would have its line near 560, a
+// condensing one near 800.  Grids so narrow that 32-wide tiles stay mostly empty have it at 6.25 loads
+// per 32 x 8 tile: 16 x 1280 cells 962 (268 / 271, 194 / 220), 4 x 5120 cells 2561 (573 / 891, 430 / 550).
+// 8 x 2 tiles up to 400 of them, 8 x 4 beyond (freezing plume 150 x 40, 380 tiles of 8 x 2: 98 / 103;
+// condensing 256 x 64, 1,024: 241 / 185).  Nozzles have one row, which leaves 32 x 8 tiles one live row
+// too (83 to 93 us up to 4,800 cells) and makes 8 x 4 tiles 8 x 2 ones; 8 x 2 / 32 x 8: 400 cells (load
+// 101) 70 / 87, 900 (227) 80 / 84, 952 (239) 90 / 85, 1,600 104 / 86, 4,800 209 / 93, 20,000 770 / 327.
+// FP32 keeps 32 x 8, so that its totals, summed in FP32 within a warp, are those of a batch's cases; the
+// autotuner may choose the small tiles there.
 static int default_shape(const ct_case* c, int precision) {
-  if (variant_of(c, precision) != 0 || cells_of(c) > SMALL_GRID) return 0;
+  if (variant_of(c, precision) != 0 || !shape_serves(10, c)) return 0;
+  const int load = num_blocks(c, 10) + tiles_x(c, 10) + tiles_y(c, 10);
+  if (case_nr(c) == 1) return load <= 230 ? 11 : 0;
+  if (load > 740 && 4 * load > 25 * num_blocks(c, 0)) return 0;
   return num_blocks(c, 11) <= 400 ? 11 : 10;
 }
 static int shape_for(const ct_case* c, int precision) {

@@ -1530,10 +1530,10 @@ struct StageSet {
   size_t queue_smem;                // their dynamic shared memory
   bool small_grid;                  // for grids of at most SMALL_GRID cells only
 };
-// Largest grid the small tiles serve, in cells.  A step of the freezing plume in FP64 on GB300, 32 x 8
-// tiles / 8 x 4 tiles: a condensing plume 256 x 64 256 / 188 us (300 x 80 cells 268 / 181 before
-// the source's shares); on 400 x 100 cells, which give every SM a 32 x 8 tile, 263 / 264 and 280 / 376
-// before them, 243 and 258 with 32 x 8 tiles now.
+// Largest grid the small tiles serve, in cells: 640 full tiles of 8 x 4, where a condensing plume still
+// gains by them (256 x 79 cells: 208 us a step, 32 x 8 tiles 257) and a dormant one no longer does (130
+// and 117); with 400 x 100 cells a condensing one lost too (376 and 280, before the source's shares).
+// Which of the smaller grids take them by default: default_shape in contrail.cu.
 constexpr size_t SMALL_GRID = 20480;
 constexpr size_t SMEM_LIMIT = 227 * 1024 - 4096;   // opt-in limit minus the static shared memory
 
