@@ -118,19 +118,16 @@ ct_status ct_mlp_infer(const void* blob, const float* X, int n, float* Y, int* e
   if (!blob || !X || !Y || !err_flag || n < 0) return ct__set_error(CT_ERR_ARG, "ct_mlp_infer: bad argument");
   if (((uintptr_t)blob & 15) != 0) return ct__set_error(CT_ERR_ARG, "ct_mlp_infer: blob must be 16-byte aligned");
   if (n == 0) return CT_OK;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GROUP_SMEM);
-    if (e != cudaSuccess) return ct__set_error(CT_ERR_CUDA, cudaGetErrorString(e));
-    attr = true;
-  }
+  // on every call: the limit belongs to the current device
+  cudaError_t e = cudaFuncSetAttribute(k_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GROUP_SMEM);
+  if (e != cudaSuccess) return ct__set_error(CT_ERR_CUDA, cudaGetErrorString(e));
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int ntiles = (n + 127) / 128;
   const int grid = ntiles < nsm ? ntiles : nsm;
   k_infer<<<grid, 128 * GROUPS, GROUP_SMEM, (cudaStream_t)stream>>>((const unsigned char*)blob, X, n, Y, err_flag);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   return e == cudaSuccess ? CT_OK : ct__set_error(CT_ERR_CUDA, cudaGetErrorString(e));
 }
 
