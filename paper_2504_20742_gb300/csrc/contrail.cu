@@ -726,12 +726,14 @@ static int queue_grid() {
 }
 
 static std::mutex g_attr_mu;
-static bool g_attr_done[NSHAPES][NVARIANT];
+static bool g_attr_done[64][NSHAPES][NVARIANT];   // per device
 
-// Opt the kernels of one (shape, kernel variant) into their dynamic shared memory, once.
+// Opt the kernels of one (shape, kernel variant) into their dynamic shared memory, once per device.
 static ct_status set_stage_attrs(int shape, int p) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return fail(CT_ERR_CUDA, "current device");
   std::lock_guard<std::mutex> lk(g_attr_mu);
-  if (g_attr_done[shape][p]) return CT_OK;
+  if (dev < 64 && g_attr_done[dev][shape][p]) return CT_OK;
   const StageSet* ss = stage_set(shape);
   cudaError_t e = cudaSuccess;
   for (int st = 0; st < 2 && e == cudaSuccess; ++st) {
@@ -749,7 +751,7 @@ static ct_status set_stage_attrs(int shape, int p) {
   if (e != cudaSuccess) return fail(CT_ERR_CUDA, cudaGetErrorString(e));
   if (p == 2 && ss->queue[0] && queue_grid() <= 0)
     return fail(CT_ERR_CUDA, "no resident CTA for the surrogate queue kernel");
-  g_attr_done[shape][p] = true;
+  if (dev < 64) g_attr_done[dev][shape][p] = true;
   return CT_OK;
 }
 

@@ -51,3 +51,21 @@ def test_training_kernels(fake, buf):
     wb = fake.ct_mlp_work_bytes(n)
     _both_devices(fake, lambda: fake.ct_mlp_loss_grad(buf, buf, buf, buf, n, buf, buf, buf, wb, None))
     _both_devices(fake, lambda: fake.ct_mlp_loss_grad_tc(buf, buf, buf, buf, n, buf, buf, buf, buf, wb, None))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_steps(fake, buf, prec):
+    from paper_2504_20742_gb300 import _lib
+    from synth import cases
+    c = _lib._case(cases.plume_case(nx=256, nr=128)[0])
+    _both_devices(fake, lambda: fake.ct_step(C.byref(c), prec, buf, buf + 64, buf, 1, 0.5, None))
+
+
+def test_surrogate_steps(fake, buf):
+    from paper_2504_20742_gb300 import _lib
+    from synth import cases
+    c = _lib._case(cases.plume_case(nx=256, nr=128)[0])
+    for shape in (0, 9):                                  # the fused tile, the column sweep and its queue
+        assert fake.ct_set_tile_shape(C.byref(c), 2, shape) == 0
+        _both_devices(fake, lambda: fake.ct_step_surrogate(C.byref(c), buf, buf + 64, buf, buf, 1, 0.5, None))
+    fake.ct_set_tile_shape(C.byref(c), 2, -1)
