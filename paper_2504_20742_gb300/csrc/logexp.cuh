@@ -33,12 +33,23 @@ __device__ __forceinline__ double f2d_bits(float x) {
   const unsigned h = (u & 0x80000000u) | ((a >> 3) + 0x38000000u);
   return __hiloint2double((int)(a >= 0x00800000u ? h : 0u), (int)(a >= 0x00800000u ? u << 29 : 0u));
 }
-// x / 2 on the integer pipe: exact for normal x with a normal half; zero, subnormal, infinite and
-// NaN values are returned as they are
+// x / 2 on the integer pipe, for zero and normal x with a normal half: what the reductions below take
+// (their r is zero or so large, or its square underflows whatever its half is)
+__device__ __forceinline__ double half_normal(double x) {
+  const int h = __double2hiint(x);
+  return __hiloint2double(((unsigned)h & 0x7ff00000u) != 0u ? h - 0x00100000 : h, __double2loint(x));
+}
+// x / 2 on the integer pipe, for every x: one off the exponent; where that ends (zero, subnormals and
+// the lowest normal binade share their scale), half of the bits, rounded to even.  Infinite and NaN
+// values are returned as they are.
 __device__ __forceinline__ double half_bits(double x) {
   const int h = __double2hiint(x);
   const unsigned e = (unsigned)h & 0x7ff00000u;
-  return __hiloint2double(e - 0x00100000u < 0x7fe00000u ? h - 0x00100000 : h, __double2loint(x));
+  if (e <= 0x00100000u) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull, q = m >> 1;
+    return __longlong_as_double((long long)((b ^ m) | (q + (m & q & 1ull))));
+  }
+  return __hiloint2double(e != 0x7ff00000u ? h - 0x00100000 : h, __double2loint(x));
 }
 
 // CUDA's functions for the other arguments, out of line: their code (some 150 instructions each) is
@@ -61,7 +72,7 @@ __device__ __forceinline__ double log_t(double x) {
   const double r = fma(m, __hiloint2double(0x3fe00000 + (k << 11), 0), -1.0);
   const float rf = d2f_bits(r);
   const float w = fmaf(rf * rf * rf, fmaf(rf, fmaf(rf, 0.2f, -0.25f), 0.33333334f), fmaf(ef, mtab::LN2_L, __ldg(mtab::LOG_LO + k)));
-  const double s = fma(-half_bits(r), r, r);
+  const double s = fma(-half_normal(r), r, r);
   const double t = fma(f2d_bits(ef), mtab::LN2_H, __ldg(mtab::LOG_HI + k));   // exact
   return t + (s + f2d_bits(w));
 }
@@ -81,7 +92,7 @@ __device__ __forceinline__ double exp_parts(double x, double& s) {
     s = fma(r * r, fma(r, 1.0 / 6.0, 0.5), r) + f2d_bits(w);
   } else {
     const float w = fmaf(rf * rf * rf, fmaf(rf, 0.041666668f, 0.16666667f), low);
-    s = fma(half_bits(r), r, r) + f2d_bits(w);
+    s = fma(half_normal(r), r, r) + f2d_bits(w);
   }
   const double T = __ldg(mtab::EXP_HI + i);
   return __hiloint2double(__double2hiint(T) + ((n >> 9) << 20), __double2loint(T));

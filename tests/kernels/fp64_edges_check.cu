@@ -1,4 +1,5 @@
-// Test kernel: the FP64 saturation temperature of the tabulated curves (physics.cuh).
+// Test kernel: the FP64 saturation temperature of the tabulated curves (physics.cuh), and logexp.cuh's
+// halving where the exponent field runs out.
 #include <cuda_runtime.h>
 
 #include "../../paper_2504_20742_gb300/csrc/physics.cuh"
@@ -10,7 +11,8 @@ __global__ void k_edges(int which, const double* __restrict__ x, const double* _
   sc.tables = 1;
   sc.tab = tab;
   if (which == 0) r[i] = ct::prop_tsat<double, false>(sc, x[i]);
-  else r[i] = ct::prop_tsat<double, true>(sc, x[i]);
+  else if (which == 1) r[i] = ct::prop_tsat<double, true>(sc, x[i]);
+  else r[i] = ct::half_bits(x[i]);
 }
 
 extern "C" int fp64_edges(int which, const double* x, const double* tab, double* r, int n) {

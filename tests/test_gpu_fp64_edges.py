@@ -1,6 +1,6 @@
 """FP64 source arithmetic where its fast forms reach the end of their range: the saturation
 temperature of the tabulated curves beyond the tables' nodes (150 to 640 K), against six Newton steps
-on the table in numpy."""
+on the table in numpy, and logexp.cuh's halving near the smallest numbers."""
 import ctypes
 import os
 import shutil
@@ -77,3 +77,17 @@ def test_tabulated_saturation_temperature_beyond_the_nodes(lib, ice):
     got = lib(ice, lnpv)
     bad = ~(np.abs(got - T) <= tol)
     assert not bad.any(), (lnpv[bad][:3], got[bad][:3], T[bad][:3])
+
+
+# An exact half, rounded to even where a subnormal's last bit goes, as the multiplication by 1/2 is.
+def test_halving_near_the_smallest_numbers(lib):
+    g = np.random.default_rng(6)
+    low = (g.integers(0, 1 << 54, 4000, dtype=np.uint64) >> g.integers(0, 54, 4000, dtype=np.uint64))   # below 2^-1020
+    x = np.concatenate([low.view(np.float64), 5e-324 * np.arange(9), 2.0 ** np.arange(-1074.0, -1015.0),
+                        [np.nextafter(2.0 ** -1021, 0), np.nextafter(2.0 ** -1022, 0), 1.7976931348623157e308, np.inf]])
+    x = np.concatenate([x, -x])
+    with np.errstate(under="ignore"):
+        want = 0.5 * x
+    got = lib(2, x)
+    assert np.array_equal(got.view(np.int64), want.view(np.int64))
+    assert np.isnan(lib(2, [np.nan])).all()
