@@ -102,7 +102,7 @@ def _workload(name):
 # moments in air without liquid or ice), and DRAM bytes per cell per launch (mean of the two stages) by tile shape,
 # reported only for a shape counted on the current kernel.
 FP64_FLOPS_PER_CELL_STAGE = 481.5
-FP64_TRAFFIC_PER_CELL_LAUNCH = {6: 399.2, 7: 455.6, 8: 397.9}    # 16 x 12, 16 x 16, 16 x 15, two CTAs per SM
+FP64_TRAFFIC_PER_CELL_LAUNCH = {6: 399.2, 7: 455.6, 12: 397.9}    # 16 x 12, 16 x 16, 16 x 15, two CTAs per SM
 FP32_TRAFFIC_PER_CELL_LAUNCH = {9: 140.4}    # the column sweep (28 x 64 strips), four CTAs per SM
 SWEEP_SHAPE = 9   # tile shape index of the column-sweep FP32 kernel (k_sweep)
 # the viscous FP64 kernel (same capture recipe, plume with nu_t = 0.5 m^2/s, 16 x 16 two-CTA tile:

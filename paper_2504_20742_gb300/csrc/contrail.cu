@@ -332,6 +332,7 @@ const StageSet* stage_set_16x16_o3();
 const StageSet* stage_set_32x8_o3();
 const StageSet* stage_set_16x12_d2();
 const StageSet* stage_set_16x16_d2();
+const StageSet* stage_set_16x14_d2();
 const StageSet* stage_set_16x15_d2();
 const StageSet* stage_set_sweep();
 const StageSet* stage_set_8x4();
@@ -345,10 +346,11 @@ const StageSet* stage_set(int shape) {
     case 5: return stage_set_32x8_o3();
     case 6: return stage_set_16x12_d2();
     case 7: return stage_set_16x16_d2();
-    case 8: return stage_set_16x15_d2();
+    case 8: return stage_set_16x14_d2();
     case 9: return stage_set_sweep();
     case 10: return stage_set_8x4();
     case 11: return stage_set_8x2();
+    case 12: return stage_set_16x15_d2();
     default: return stage_set_32x8();
   }
 }

@@ -1637,10 +1637,10 @@ StageSet make_stage_set_small() {
 }
 
 // the tile shapes the library is built with (one translation unit each)
-constexpr int NSHAPES = 12;
+constexpr int NSHAPES = 13;
 // 0: 32x8, 1: 16x16, 2: 32x16, 3: 64x8, 4: 16x16 and 5: 32x8 with three FP32 CTAs per SM, 6: 16x12,
-// 7: 16x16 and 8: 16x15 with two FP64 CTAs per SM, 9: the column sweep, 10: 8x4 and 11: 8x2 for
-// small grids
+// 7: 16x16 and 8: 16x14 with two FP64 CTAs per SM, 9: the column sweep, 10: 8x4 and 11: 8x2 for
+// small grids, 12: 16x15 with two FP64 CTAs per SM.  Callers keep these numbers: a new shape goes at the end.
 const StageSet* stage_set(int shape);
 
 }  // namespace ct
