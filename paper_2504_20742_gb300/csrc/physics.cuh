@@ -232,23 +232,16 @@ __device__ __forceinline__ bool moments_zero(const Get& got) {
 
 // BI: the state has the 18 fields of the bimodal liquid; Y_l is the sum of both sets.
 // Every operation has its rounding pinned: the primitive variables a kernel stores for the
-// next stage are then bit for bit those the next stage would compute itself.  ZERO: the
-// moment fields are +-0 (no liquid, no ice), and the terms they enter drop out exactly
-// (x - 0 = x, fma(0, c, x) = x for x != 0, and (+-0) / rho keeps the zero's sign), so the
-// same bits come with fewer operations.
-template <class T, bool BI, bool ZERO>
-__device__ __forceinline__ void cons_to_prim_impl(const T* U, Prim<T>& w) {
+// next stage are then bit for bit those the next stage would compute itself.
+template <bool BI>
+__device__ __forceinline__ void cons_to_prim32(const float* U, Prim<float>& w) {
+  using T = float;
   const T rho = U[0];
   // rho c_v straight from the conserved partial densities, then one reciprocal serves
   // 1/rho = (rho c_v) X and 1/c_v = rho^2 X, X = 1/(rho rho c_v)
-  T rcv;
-  if constexpr (ZERO) {
-    rcv = rn_fma(U[4], T(k::CVV), rn_mul(rn_sub(rho, U[4]), T(k::CVA)));
-  } else {
-    const T rYl = rn_mul(T(k::YL3), BI ? rn_add(U[8], U[17]) : U[8]), rYs = rn_mul(T(k::YS3), U[12]);
-    const T rYa = rn_sub(rn_sub(rn_sub(rho, U[4]), rYl), rYs);
-    rcv = rn_fma(rYs, T(k::CS), rn_fma(rYl, T(k::CL), rn_fma(U[4], T(k::CVV), rn_mul(rYa, T(k::CVA)))));
-  }
+  const T rYl = rn_mul(T(k::YL3), BI ? rn_add(U[8], U[17]) : U[8]), rYs = rn_mul(T(k::YS3), U[12]);
+  const T rYa = rn_sub(rn_sub(rn_sub(rho, U[4]), rYl), rYs);
+  const T rcv = rn_fma(rYs, T(k::CS), rn_fma(rYl, T(k::CL), rn_fma(U[4], T(k::CVV), rn_mul(rYa, T(k::CVA)))));
   const T X = trcp(rn_mul(rho, rcv));
   const T ir = rn_mul(rcv, X);
   w.rho = rho;
@@ -257,32 +250,32 @@ __device__ __forceinline__ void cons_to_prim_impl(const T* U, Prim<T>& w) {
   w.Yv = rn_mul(U[4], ir);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    w.ml[q] = ZERO ? U[5 + q] : rn_mul(U[5 + q], ir);
-    w.ms[q] = ZERO ? U[9 + q] : rn_mul(U[9 + q], ir);
+    w.ml[q] = rn_mul(U[5 + q], ir);
+    w.ms[q] = rn_mul(U[9 + q], ir);
   }
   w.ns = rn_mul(U[13], ir);
   if constexpr (BI) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) w.mh[q] = ZERO ? U[14 + q] : rn_mul(U[14 + q], ir);
+    for (int q = 0; q < 4; ++q) w.mh[q] = rn_mul(U[14 + q], ir);
     w.Yl = rn_mul(T(k::YL3), rn_add(w.ml[3], w.mh[3]));
   } else {
-    w.Yl = ZERO ? w.ml[3] : rn_mul(T(k::YL3), w.ml[3]);
+    w.Yl = rn_mul(T(k::YL3), w.ml[3]);
   }
-  w.Ys = ZERO ? w.ms[3] : rn_mul(T(k::YS3), w.ms[3]);
-  const T Ya = ZERO ? rn_sub(T(1), w.Yv) : rn_sub(rn_sub(rn_sub(T(1), w.Yv), w.Yl), w.Ys);
+  w.Ys = rn_mul(T(k::YS3), w.ms[3]);
+  const T Ya = rn_sub(rn_sub(rn_sub(T(1), w.Yv), w.Yl), w.Ys);
   const T ke = rn_mul(T(0.5), rn_fma(w.u, w.u, rn_mul(w.v, w.v)));
   const T e = rn_fma(U[3], ir, -ke);
   w.cv = rn_mul(rcv, ir);
   const T icv = rn_mul(rn_mul(rho, rho), X);
-  w.Tg = ZERO ? rn_mul(rn_fma(-w.Yv, T(k::E0V), e), icv)
-              : rn_mul(rn_fma(-w.Ys, T(k::E0S), rn_fma(-w.Yv, T(k::E0V), e)), icv);
+  w.Tg = rn_mul(rn_fma(-w.Ys, T(k::E0S), rn_fma(-w.Yv, T(k::E0V), e)), icv);
   w.Rg = rn_fma(w.Yv, T(k::RV), rn_mul(Ya, T(k::RA)));
   w.p = rn_mul(rn_mul(rho, w.Rg), w.Tg);
   w.c2 = rn_mul(rn_mul(rn_fma(w.Rg, icv, T(1)), w.p), ir);
 }
 // FP64: the mixture's constants as differences from dry air's, one operation per constituent, and
-// halves on the integer pipe (the FP64 pipe bounds the FP64 kernels); the same bits with and
-// without ZERO as above.
+// halves on the integer pipe (the FP64 pipe bounds the FP64 kernels).  ZERO: the moment fields are +-0
+// (no liquid, no ice), and the terms they enter drop out exactly (x - 0 = x, fma(0, c, x) = x for
+// x != 0, and (+-0) / rho keeps the zero's sign), so the same bits come with fewer operations.
 template <bool BI, bool ZERO>
 __device__ __forceinline__ void cons_to_prim64(const double* U, Prim<double>& w) {
   const double rho = U[0];
@@ -334,7 +327,7 @@ __device__ __forceinline__ void cons_to_prim(const T* U, Prim<T>& w) {
     else
       cons_to_prim64<BI, false>(U, w);
   } else {
-    cons_to_prim_impl<T, BI, false>(U, w);
+    cons_to_prim32<BI>(U, w);
   }
 }
 
