@@ -102,7 +102,7 @@ def _workload(name):
 # moments in air without liquid or ice), and DRAM bytes per cell per launch (mean of the two stages) by tile shape,
 # reported only for a shape counted on the current kernel.
 FP64_FLOPS_PER_CELL_STAGE = 481.5
-FP64_TRAFFIC_PER_CELL_LAUNCH = {6: 399.2, 7: 455.6, 12: 397.9}    # 16 x 12, 16 x 16, 16 x 15, two CTAs per SM
+FP64_TRAFFIC_PER_CELL_LAUNCH = {6: 399.2, 7: 455.6, 8: 395.5, 12: 397.9}    # 16 x 12, 16 x 16, 16 x 14, 16 x 15, two CTAs per SM
 FP32_TRAFFIC_PER_CELL_LAUNCH = {9: 140.4}    # the column sweep (28 x 64 strips), four CTAs per SM
 SWEEP_SHAPE = 9   # tile shape index of the column-sweep FP32 kernel (k_sweep)
 # the viscous FP64 kernel (same capture recipe, plume with nu_t = 0.5 m^2/s, 16 x 16 two-CTA tile:
@@ -300,7 +300,7 @@ def run_cuda(args):
                 "kernel": "ct::k_stage<double>",
                 "peak_source": "measured: cuBLAS DGEMM 4096^3 on this GPU (FP64 has no entry in MEASURED_PEAKS.json)",
                 "note": f"{per_cell} FP64 flops per cell-stage executed (a DFMA counts 2, a DADD or DMUL 1; "
-                        "the FP64 pipe was 75-76 % busy on the plume in the ncu capture, profiles/); "
+                        "the FP64 pipe was 75-79 % busy on the plume in the ncu capture, profiles/); "
                         "the peak is cuBLAS DGEMM timed in this run; traffic (DRAM bytes of the ncu capture) "
                         "exceeds the 280 algorithmic bytes per cell-launch because the kernel reads and "
                         "writes the stored primitive planes on purpose (DRAM 2-3 % busy); "
